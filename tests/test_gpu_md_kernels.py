@@ -1,0 +1,61 @@
+"""Gauge force, plaquette and link update at the edges of their work split: lattices
+that fill a fraction of a block, one block and a ragged last block, momenta on
+either side of the exponential's degree and scaling thresholds, and matrices
+that are not Hermitian."""
+import numpy as np
+import pytest
+
+from oracle import gauge as og
+from synthetic import gauge_field, make_rng, random_su3_algebra
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def L():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1512_03487_gb300 as L
+    from paper_1512_03487_gb300 import fields
+    L.fields = fields
+    return L
+
+
+def _rel(a, b):
+    return float(np.abs(a - b).max() / np.abs(b).max())
+
+
+# sums of at most some hundred products of entries below 1: 1e-13 is about 500 roundings
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (2, 2, 2, 4), (4, 2, 2, 6), (6, 2, 10, 2)])
+def test_gauge_force_and_plaquette_on_ragged_blocks(L, dims):
+    F = L.fields
+    lat = L.lattice(dims)
+    U = gauge_field(dims, "haar", 1801)
+    U *= 1.0 + 0.1 * make_rng(1802).standard_normal(U.shape)  # the formulas hold for any matrices
+    Ud = F.gauge_to_device(U, lat, 0, 18)
+    out = torch.full((L.lqcd_gauge_bytes(lat, 0, 18),), 0xff, dtype=torch.uint8, device="cuda")
+    L.lqcd_gauge_force(out, Ud, lat, 5.6)
+    assert _rel(F.gauge_to_host(out, lat, 0, 18), og.force(U, 5.6)) <= 1e-13
+    ws = F.empty(L.lqcd_reduce_workspace_bytes(lat))
+    assert L.lqcd_plaquette(Ud, lat, ws) == pytest.approx(og.mean_plaquette(U), rel=1e-13, abs=1e-14)
+
+
+# |A|_F against the thresholds 1/4 (degree 13 or 20) and 1 (halvings); at 6 there
+# are three squarings, each doubling some tens of roundings: below 1e-13
+@pytest.mark.parametrize("norm", [0.0, 0.2499, 0.2501, 0.9999, 1.0001, 6.0])
+@pytest.mark.parametrize("hermitian", [True, False])
+def test_link_update_around_its_thresholds(L, norm, hermitian):
+    from scipy.linalg import expm
+    F = L.fields
+    dims = (4, 2, 2, 2)
+    lat = L.lattice(dims)
+    U = gauge_field(dims, "haar", 1811)
+    n = U.size // 9
+    rng = make_rng(1812)
+    P = random_su3_algebra(rng, n) if hermitian else rng.standard_normal((n, 3, 3)) + 1j * rng.standard_normal((n, 3, 3))
+    P *= (norm / 0.5 / np.linalg.norm(P, axis=(1, 2)))[:, None, None]
+    expect = np.einsum("nij,njk->nik", np.stack([expm(0.5j * p) for p in P]), U.reshape(n, 3, 3)).reshape(U.shape)
+    Ud = F.gauge_to_device(U, lat, 0, 18)
+    L.lqcd_gauge_exp_update(Ud, F.gauge_to_device(P.reshape(U.shape), lat, 0, 18), 0.5, lat)
+    assert _rel(F.gauge_to_host(Ud, lat, 0, 18), expect) <= 1e-13
