@@ -1,12 +1,14 @@
-"""Gauge force, plaquette and link update at the edges of their work split: lattices
+"""Gauge force, fermion force, plaquette and link update at the edges of their work split: lattices
 that fill a fraction of a block, one block and a ragged last block, momenta on
 either side of the exponential's degree and scaling thresholds, and matrices
 that are not Hermitian."""
 import numpy as np
 import pytest
 
+from oracle import force as oforce
 from oracle import gauge as og
-from synthetic import gauge_field, make_rng, random_su3_algebra
+from synthetic import gauge_field, gaussian_spinor, make_rng, random_su3_algebra
+from tests.layout import rel_l2
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -59,3 +61,21 @@ def test_link_update_around_its_thresholds(L, norm, hermitian):
     Ud = F.gauge_to_device(U, lat, 0, 18)
     L.lqcd_gauge_exp_update(Ud, F.gauge_to_device(P.reshape(U.shape), lat, 0, 18), 0.5, lat)
     assert _rel(F.gauge_to_host(Ud, lat, 0, 18), expect) <= 1e-13
+
+
+# sums of at most a hundred products, as in the oracle: 1e-12 as for the full lattices
+@pytest.mark.parametrize("recon", [18, 12])
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (4, 2, 2, 2), (2, 6, 2, 6)])
+def test_fermion_force_on_ragged_blocks(L, dims, recon):
+    F = L.fields
+    bc = (1.0, -1.0, 1.0, -1.0)
+    U, X, Y = gauge_field(dims, "haar", 1821), gaussian_spinor(dims, 1822), gaussian_spinor(dims, 1823)
+    lat = L.lattice(dims, bc=bc)
+    op = L.operator(mass=0.05, recon=recon)
+    g = F.gauge_to_device(U, lat, 0, recon)
+    Xd, Yd = (F.spinor_to_device(f[None], lat, 0, 2) for f in (X, Y))
+    grad, ta = oforce.force_terms(U, X, Y, bc)
+    for kind, ref in ((L.LQCD_FORCE_TA, ta), (L.LQCD_FORCE_GRAD, grad)):
+        out = torch.full((L.lqcd_gauge_bytes(lat, 0, 18),), 0xff, dtype=torch.uint8, device="cuda")
+        L.lqcd_force(out, g, Xd, Yd, lat, op, kind)
+        assert rel_l2(F.gauge_to_host(out, lat, 0, 18), ref) <= 1e-12
