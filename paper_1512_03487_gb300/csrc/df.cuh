@@ -80,20 +80,16 @@ __device__ __forceinline__ dfl fma(dfl a, dfl b, dfl c) { return df_fma(a, b, c)
 // bits: hi's exponent is rebased from the FP64 bias 1023 to the FP32 bias 127
 // and its mantissa is the top 23 stored bits; lo = m29 2^-52 2^(e - 1023) with
 // the sign of the double (both factors are normal floats over hi's range, so lo
-// underflows only gradually, where |lo| < 2^-126). |d| below 2^-126 (FP32's
-// normal range) splits to zero; |d| must stay below 2^128.
+// underflows only gradually, where |lo| < 2^-126): six integer instructions, a
+// conversion and two products. |d| below 2^-126 (FP32's normal range) splits to a
+// value below 2^-126, zero to zero; |d| must stay below 2^128.
 __device__ __forceinline__ dfl df_split(double d) {
   const unsigned int hw = (unsigned int)__double2hiint(d);
   const unsigned int lw = (unsigned int)__double2loint(d);
-  const unsigned int e = (hw >> 20) & 0x7ffu;
-  const unsigned int sign = hw & 0x80000000u;
-  unsigned int hb = __funnelshift_l(lw, hw - (896u << 20), 3);
-  hb = (hb & 0x7fffffffu) | sign;
+  const unsigned int t = (unsigned int)__viaddmax_s32((int)(hw & 0x7fffffffu), -(896 << 20), 0);
+  const unsigned int hb = __funnelshift_l(lw, t, 3) | (hw & 0x80000000u);
   const float m = __fmul_rn((float)(lw & 0x1fffffffu), 0x1p-52f);
-  const float scale = __int_as_float((int)((e - 896u) << 23));  // 2^(e - 1023), normal for 897 <= e <= 1150
-  const float lo = __int_as_float(__float_as_int(__fmul_rn(m, scale)) | (int)sign);
-  const bool normal = e >= 897u;
-  return dfl(normal ? __int_as_float((int)hb) : 0.f, normal ? lo : 0.f);
+  return dfl(__uint_as_float(hb), __fmul_rn(m, __uint_as_float(hb & 0xff800000u)));  // +- 2^(e - 1023)
 }
 
 __device__ __forceinline__ dfl::dfl(double d) {

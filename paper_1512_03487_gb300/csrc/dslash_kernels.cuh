@@ -342,113 +342,6 @@ struct EpiCoef {
   double a, b, m5d, mf;
 };
 
-// ---- the hop with its eight directions in a rolled loop (runtime mu): one copy
-// of the per-direction code instead of eight. For the double-float arithmetic a
-// fully unrolled hop is about 19,000 instructions long and stalls on
-// instruction fetch; this form keeps the loop body in the instruction cache.
-
-// z times c, c = +-1 or +-i: imag selects i, neg the sign
-template <typename T> __device__ __forceinline__ cpx<T> times_unit(cpx<T> z, bool imag, bool neg) {
-  const cpx<T> r = imag ? mk(-z.i, z.r) : z;
-  return neg ? mk(-r.r, -r.i) : r;
-}
-
-// The link of direction mu into w: U (forward hop, block blk at checkerboard site
-// cb) or U^dag (backward), as the matrix U' with w = U' h. 18-real links are read
-// in the transposed order for U^dag; 12-real ones are rebuilt, then transposed.
-template <int P, int R>
-__device__ __forceinline__ void load_link_rolled(const void* gauge, int64_t gs, int blk, int64_t cb, bool fwd,
-                                                 Link<typename PrecTraits<P>::real>& u) {
-  using T = typename PrecTraits<P>::real;
-  if constexpr (R == 18) {
-    const double2* b = reinterpret_cast<const double2*>(gauge) + (int64_t)blk * 9 * gs + cb;
-    static_assert(P == LQCD_F64 || P == LQCD_F64_DF, "rolled hop: FP64 fields");
-#pragma unroll
-    for (int r = 0; r < 3; r++)
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        const double2 w = __ldg(b + (fwd ? 3 * r + c : 3 * c + r) * gs);
-        const double im = fwd ? w.y : -w.y;
-        if constexpr (P == LQCD_F64_DF) u.v[3 * r + c] = mk(df_split(w.x), df_split(im));
-        else u.v[3 * r + c] = mk(w.x, im);
-      }
-  } else {
-    Link<T> v;
-    LinkIO<P, 12>::load(gauge, gs, blk, cb, v);
-#pragma unroll
-    for (int r = 0; r < 3; r++)
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        const cpx<T> a = v.v[3 * r + c], t = conj(v.v[3 * c + r]);
-        u.v[3 * r + c] = fwd ? a : t;
-      }
-  }
-}
-
-template <int P, int R, bool DAG>
-__device__ __forceinline__ void hop_acc_rolled(const Geom& g, const void* gauge, const void* in, int parity,
-                                               int64_t j, Spinor<typename PrecTraits<P>::real>& acc) {
-  using T = typename PrecTraits<P>::real;
-  const int64_t n5 = g.n5;
-  int64_t cb, i5;
-  if (n5 == 1) {
-    cb = j;
-    i5 = 0;
-  } else {
-    cb = fdiv((uint32_t)j, g.fn5);
-    i5 = j - cb * n5;
-  }
-  const Coord x = cb_to_coord(g, cb, parity);
-  zero(acc);
-  constexpr int SF = DAG ? +1 : -1;  // forward hop carries (1 + SF gamma_mu)
-#pragma unroll 1
-  for (int dir = 0; dir < 8; dir++) {
-    const int mu = dir >> 1;
-    const bool fwd = (dir & 1) == 0;
-    const bool sneg = (fwd ? SF : -SF) < 0;  // the projector's sign S is -1
-    // neighbour along +-mu
-    const int L = mu == 0 ? g.X : mu == 1 ? g.Y : mu == 2 ? g.Z : g.T;
-    const int xm = mu == 0 ? x.c[0] : mu == 1 ? x.c[1] : mu == 2 ? x.c[2] : x.c[3];
-    const uint32_t st = mu == 0 ? 1u : mu == 1 ? (uint32_t)g.st[1] : mu == 2 ? (uint32_t)g.st[2] : (uint32_t)g.st[3];
-    const bool wrap = fwd ? xm == L - 1 : xm == 0;
-    const uint32_t lex = fwd ? (wrap ? x.lex - (uint32_t)(L - 1) * st : x.lex + st)
-                             : (wrap ? x.lex + (uint32_t)(L - 1) * st : x.lex - st);
-    const int64_t nb = (int64_t)(lex >> 1);
-    Spinor<T> p;
-    SpinorIO<P>::load(in, g.sstride, nb * n5 + i5, p);
-    // (1 + S gamma_mu) in the chiral basis: h0 = p0 + c0 p_k0, h1 = p1 + c1 p_k1 with
-    // c = sc S (i if mu is even), and the lower spins S B^dag w: spin 2 += d2 w_m2,
-    // spin 3 += d3 w_m3 with d = sd S (i if mu is even)
-    const bool imag = (mu & 1) == 0;
-    const bool k0_is3 = mu < 2;
-    const bool c0neg = (mu != 3) != sneg, c1neg = (mu == 0) != sneg;
-    const bool d2neg = sneg, d3neg = (mu == 1 || mu == 2) != sneg;
-    Half<T> h;
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-      const cpx<T> a0 = k0_is3 ? p.v[9 + c] : p.v[6 + c];
-      const cpx<T> a1 = k0_is3 ? p.v[6 + c] : p.v[9 + c];
-      h.v[c] = p.v[c] + times_unit(a0, imag, c0neg);
-      h.v[3 + c] = p.v[3 + c] + times_unit(a1, imag, c1neg);
-    }
-    Link<T> u;
-    load_link_rolled<P, R>(gauge, g.gstride, fwd ? parity * 4 + mu : (1 - parity) * 4 + mu, fwd ? cb : nb, fwd, u);
-    Half<T> w;
-    link_mul(u, h, w);
-    // a wrapping hop's boundary phase (+-1) flips the signs of its whole contribution
-    const float bcm = mu == 0 ? g.bcf[0] : mu == 1 ? g.bcf[1] : mu == 2 ? g.bcf[2] : g.bcf[3];
-    const bool pneg = wrap && bcm < 0.f;
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-      const cpx<T> w0 = w.v[c], w1 = w.v[3 + c];
-      acc.v[c] = acc.v[c] + times_unit(w0, false, pneg);
-      acc.v[3 + c] = acc.v[3 + c] + times_unit(w1, false, pneg);
-      acc.v[6 + c] = acc.v[6 + c] + times_unit(k0_is3 ? w1 : w0, imag, d2neg != pneg);
-      acc.v[9 + c] = acc.v[9 + c] + times_unit(k0_is3 ? w0 : w1, imag, d3neg != pneg);
-    }
-  }
-}
-
 // Both hops along mu with spin-paired packed arithmetic (hop_pair.cuh): the
 // projection and the link as in hop_dir, the products and the accumulation on
 // (spin 0, spin 1) pairs. FP32 / FP16 storage, no G-parity.
@@ -488,6 +381,7 @@ __device__ __forceinline__ void hop_dir_sp(SPAcc& acc, const Geom& g, const void
 }  // namespace lqcd
 
 #include "hop_async.cuh"  // the staged hop uses the projections and products above
+#include "hop_df.cuh"
 
 namespace lqcd {
 
@@ -498,7 +392,10 @@ __device__ __forceinline__ void hop_acc(const Geom& g, const void* gauge, const 
                                         Spinor<typename PrecTraits<P>::real>& acc,
                                         const Link<typename PrecTraits<P>::real>* sl = nullptr,
                                         unsigned char* ring = nullptr) {
-  if constexpr (AS) {
+  if constexpr (P == LQCD_F64_DF) {
+    hop_acc_df<R, DAG, AS, BLOCK>(g, gauge, in, parity, j, acc, ring);
+    return;
+  } else if constexpr (AS) {
     hop_acc_async<P, R, DAG, SP, BLOCK>(g, gauge, in, parity, j, acc, ring);
     return;
   }
@@ -510,10 +407,6 @@ __device__ __forceinline__ void hop_acc(const Geom& g, const void* gauge, const 
   } else {
     cb = fdiv((uint32_t)j, g.fn5);
     i5 = j - cb * n5;
-  }
-  if constexpr (P == LQCD_F64_DF) {
-    hop_acc_rolled<P, R, DAG>(g, gauge, in, parity, j, acc);
-    return;
   }
   const Coord x = cb_to_coord(g, cb, parity);
   if constexpr (SP) {
@@ -642,6 +535,12 @@ __device__ __forceinline__ void stage_links(const Geom& g, const void* gauge, in
   __syncthreads();
 }
 
+// Shared memory of a hop whose neighbour data are copied asynchronously (AS)
+template <int P, int R> constexpr int ring_bytes(int block) {
+  if constexpr (P == LQCD_F64_DF) return df_ring_bytes<R>(block);
+  else return stage_nslot<P>() * stage_slot_bytes<P, R>() * block;
+}
+
 // One launch computes BLOCK * SPT output sites per block. SPT = 1: one site
 // per thread, any precision. SPT = 2 (FP32 and FP16 storage, not G-parity):
 // thread t of block blk computes sites j0 = blk BLOCK 2 + t and j1 = j0 +
@@ -682,7 +581,7 @@ __device__ __forceinline__ void hop_body(const HopArgs& A) {
     // AS: the ring of asynchronously copied neighbour data
     unsigned char* ring = nullptr;
     if constexpr (AS) {
-      __shared__ __align__(16) unsigned char stage_ring[stage_nslot<P>() * stage_slot_bytes<P, R>() * BLOCK];
+      __shared__ __align__(16) unsigned char stage_ring[ring_bytes<P, R>(BLOCK)];
       ring = stage_ring;
     }
     if constexpr (EPI == EPI_M5INV) {

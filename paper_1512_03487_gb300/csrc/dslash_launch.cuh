@@ -41,7 +41,9 @@ static int launch_hop_index(int idx, const HopArgs& a, cudaStream_t s) {
 // that may be timed (see TuningPass), else the default shape.
 template <int P, int R, bool DAG, int EPI, int RED, bool GP>
 static int launch_hop_inst(const HopArgs& a, cudaStream_t s) {
-  if constexpr (P == LQCD_F64 || P == LQCD_F64_DF || GP) {
+  if constexpr (P == LQCD_F64_DF) {
+    return launch_hop_shape<P, R, DAG, EPI, RED, GP, HOP_BLOCK, -3, 4>(a, s);
+  } else if constexpr (P == LQCD_F64 || GP) {
     return launch_hop_shape<P, R, DAG, EPI, RED, GP, HOP_BLOCK, 1, 0>(a, s);
   } else {
     const HopKey k{P, R, DAG ? 1 : 0, EPI, RED, a.full, a.g.X, a.g.Y, a.g.Z, a.g.T, a.g.n5};
