@@ -242,36 +242,90 @@ __global__ void __launch_bounds__(MG_BLOCK) k_block_orth(void* vecs, MGGeom m) {
   }
 }
 
-// c(X)[(s, k)] = sum_{x in X} P_k(x)|_s^dag psi(x)|_s; one CTA per (aggregate X, vector k)
-template <int P>
-__global__ void __launch_bounds__(MG_BLOCK) k_restrict(void* coarse, const void* fine, const void* vecs, MGGeom m) {
+// Sums of the restriction: FP32 fields add theirs up as double-float pairs, FP64 fields
+// in FP64. FP64 additions run at 1/64 of the FP32 rate (they were 71 % of the FP64
+// pipe's time when FP32 terms were summed in FP64), and the 48 bits of a pair are far
+// below the FP32 rounding of the terms and of the result.
+template <typename T> struct SumOf;
+template <> struct SumOf<float> { using type = dfl; };
+template <> struct SumOf<double> { using type = double; };
+__device__ __forceinline__ dfl xor_lanes(dfl v, int o) {
+  return dfl(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
+}
+__device__ __forceinline__ double xor_lanes(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ double sum_value(dfl v) { return df_to_double(v); }
+__device__ __forceinline__ double sum_value(double v) { return v; }
+__device__ __forceinline__ dfl add_term(dfl s, float v) {
+  float h, e;
+  two_sum(s.hi, v, h, e);
+  return fast_two_sum(h, e + s.lo);
+}
+__device__ __forceinline__ double add_term(double s, double v) { return s + v; }
+
+// c(X)[(s, k)] = sum_{x in X} P_k(x)|_s^dag psi(x)|_s. One thread per fine site, 256
+// sites per block (one aggregate of 4^4 or 16 of 2^4), all vectors: psi is read once
+// instead of once per vector, which leaves the vectors' own bytes as the floor. Four
+// vectors at a time give 16 terms per thread (two chiralities, real and imaginary)
+// that go to shared memory; then each thread adds up 16 of them.
+// 24^3 x 48, 12 FP32 vectors, 4^4 aggregates on GB300: 516 -> 171 us, 0.72 of the
+// measured copy bandwidth.
+constexpr int RS_BLOCK = 256;
+template <int P, int B>
+__global__ void __launch_bounds__(RS_BLOCK, P == LQCD_F32 ? 4 : 1) k_restrict(void* coarse, const void* fine,
+                                                                              const void* vecs, MGGeom m) {
   using T = typename PrecTraits<P>::real;
-  __shared__ double2 sh[2 * (MG_BLOCK / 32)];
-  const int64_t agg = blockIdx.x;
-  const int k = blockIdx.y;
-  const bool act = threadIdx.x < m.b * m.b * m.b * m.b;
+  using S = typename SumOf<T>::type;
+  constexpr int SITES = B * B * B * B;
+  // the 16 terms of a thread, a pitch that spreads the reads below over the banks;
+  // two buffers (FP32), so that one barrier per group is enough
+  constexpr int PITCH = B == 4 ? RS_BLOCK + 16 : RS_BLOCK + 1, BUFS = P == LQCD_F32 ? 2 : 1;
+  __shared__ T sh[BUFS][16 * PITCH];
+  const int tid = threadIdx.x;
+  const int64_t agg = (int64_t)blockIdx.x * (RS_BLOCK / SITES) + tid / SITES;
+  const bool act = agg < m.Vc;  // past the end: aggregate 0, nothing stored
   int c[4], parity;
   int64_t cb;
-  agg_site(m, agg, act ? threadIdx.x : 0, c, parity, cb);
+  agg_site(m, act ? agg : 0, tid % SITES, c, parity, cb);
   Spinor<T> psi;
-  zero(psi);
-  if (act) SpinorIO<P>::load(fine_ptr<P>(fine, m, 0, parity), m.g.sstride, cb, psi);
-  cpx<T>* out = static_cast<cpx<T>*>(coarse) + agg * m.nc;
-  Spinor<T> v;
-  zero(v);
-  if (act) SpinorIO<P>::load(fine_ptr<P>(vecs, m, k, parity), m.g.sstride, cb, v);
-  T pr[2] = {T(0), T(0)}, pi[2] = {T(0), T(0)};
+  SpinorIO<P>::load(fine_ptr<P>(fine, m, 0, parity), m.g.sstride, cb, psi);
+  T* out = static_cast<T*>(coarse);
+  // 4^4: thread t sums value t / 16 over the sites t % 16 + 16 i and meets 15 others;
+  // 2^4: thread t sums value t % 16 of its aggregate t / 16
+  const int val = B == 4 ? tid >> 4 : tid & 15, start = B == 4 ? tid & 15 : tid & ~15, stride = B == 4 ? 16 : 1;
+  for (int k0 = 0; k0 < m.nv; k0 += 4) {
+    T* buf = sh[BUFS == 2 ? (k0 >> 2) & 1 : 0];
+#pragma unroll 1  // one vector's registers: 32 warps per SM keep more loads in flight than unrolling does
+    for (int q = 0; q < 4; q++) {
+      T re[2] = {T(0), T(0)}, im[2] = {T(0), T(0)};
+      if (k0 + q < m.nv) {
+        Spinor<T> v;
+        SpinorIO<P>::load(fine_ptr<P>(vecs, m, k0 + q, parity), m.g.sstride, cb, v);
 #pragma unroll
-  for (int e = 0; e < 12; e++) {
-    const int s = e / 6;
-    pr[s] = fma(v.v[e].r, psi.v[e].r, fma(v.v[e].i, psi.v[e].i, pr[s]));
-    pi[s] = fma(v.v[e].r, psi.v[e].i, fma(-v.v[e].i, psi.v[e].r, pi[s]));
-  }
-  double2 d[2] = {make_double2((double)pr[0], (double)pi[0]), make_double2((double)pr[1], (double)pi[1])};
-  block_sum<2>(d, sh);
-  if (threadIdx.x == 0) {
-    out[k] = mk((T)d[0].x, (T)d[0].y);
-    out[m.nv + k] = mk((T)d[1].x, (T)d[1].y);
+        for (int e = 0; e < 12; e++) {
+          const int h = e / 6;
+          re[h] = fma(v.v[e].r, psi.v[e].r, fma(v.v[e].i, psi.v[e].i, re[h]));
+          im[h] = fma(v.v[e].r, psi.v[e].i, fma(-v.v[e].i, psi.v[e].r, im[h]));
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < 2; h++) {
+        buf[(4 * q + 2 * h) * PITCH + tid] = re[h];
+        buf[(4 * q + 2 * h + 1) * PITCH + tid] = im[h];
+      }
+    }
+    __syncthreads();
+    S s = S(0);
+#pragma unroll
+    for (int i = 0; i < 16; i++) s = add_term(s, buf[val * PITCH + start + i * stride]);
+    if (BUFS == 1) __syncthreads();
+    if (B == 4) {
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) s = s + xor_lanes(s, o);
+    }
+    // value: vector k0 + val / 4, chirality (val / 2) % 2, real or imaginary part
+    const int k = k0 + (val >> 2);
+    if (act && k < m.nv && (B == 2 || (tid & 15) == 0))
+      out[(agg * m.nc + ((val >> 1) & 1) * m.nv + k) * 2 + (val & 1)] = (T)sum_value(s);
   }
 }
 
@@ -319,12 +373,77 @@ __device__ __forceinline__ int64_t coarse_nb(const MGGeom& m, int64_t X, int d) 
   return cc[0] + (int64_t)m.cX * (cc[1] + (int64_t)m.cY * (cc[2] + (int64_t)m.cZ * cc[3]));
 }
 
-// out(X)_i = sum_d sum_j Y_d(X)_ij in(X + d)_j; dagger: sum_d sum_j conj(Y_{-d}(X + d)_ji) in(X + d)_j.
-// One warp per (coarse site, row): the lanes take the 9 Nc products in turn
-// (consecutive j for consecutive lanes) and the warp sums them.
+// out(X)_i = sum_d sum_j Y_d(X)_ij in(X + d)_j. Four lanes per row, eight rows of
+// one coarse site per warp (consecutive in memory): each lane takes every fourth
+// 16-byte piece of its row of the nine blocks, one load of Y, one (cached) of in
+// and their FMAs. Y is read once, and its bytes are the floor. NP: pieces per lane
+// and block, unrolled so that the loads of several blocks are in flight; 0 for row
+// lengths that are not a multiple of four pieces, or long. 2,592 sites of 24 x 24
+// blocks in FP32 on GB300: 55 -> 30 us (before: one warp per row, divisions per product).
+constexpr int CA_LANES = 4;
+template <typename T, int NP>
+__global__ void __launch_bounds__(MG_BLOCK) k_coarse_apply(cpx<T>* out, const cpx<T>* in, const cpx<T>* Y, MGGeom m) {
+  constexpr int PER = 16 / (int)sizeof(cpx<T>);  // complex values per 16-byte piece
+  struct alignas(16) Piece { cpx<T> v[PER]; };
+  using S = typename SumOf<T>::type;
+  const int nc = m.nc, rows = 32 / CA_LANES, groups = (nc + rows - 1) / rows;
+  const int wid = (int)(((int64_t)blockIdx.x * MG_BLOCK + threadIdx.x) >> 5);  // below Vc groups < 2^31
+  const int lane = threadIdx.x & 31;
+  if (wid >= m.Vc * groups) return;  // whole warps exit together
+  const int X = wid / groups;
+  const int i = (wid - X * groups) * rows + lane / CA_LANES, l = lane % CA_LANES;
+  int nb_l = X;  // lanes 1..8 find the stencil's neighbours (32-bit index arithmetic)
+  {
+    const int mu = (lane - 1) >> 1, stx = m.cX, sty = stx * m.cY, stz = sty * m.cZ;
+    const int L = mu == 0 ? m.cX : mu == 1 ? m.cY : mu == 2 ? m.cZ : m.cT;
+    const int st = mu == 0 ? 1 : mu == 1 ? stx : mu == 2 ? sty : stz;
+    const int at = X / st % L;
+    if (lane > 0 && lane < 9)
+      nb_l += (lane & 1) ? (at == L - 1 ? -(L - 1) * st : st) : (at == 0 ? (L - 1) * st : -st);
+  }
+  const int pieces = nc / PER;
+  const int64_t block = (int64_t)nc * nc;
+  const Piece* y = reinterpret_cast<const Piece*>(Y + X * block + (int64_t)(i < nc ? i : 0) * nc) + l;
+  const int64_t ystep = m.Vc * block / PER;
+  // a block's products in T, the sum over the blocks and lanes as in the restriction
+  S sr = S(0), si = S(0);
+#pragma unroll
+  for (int d = 0; d < 9; d++) {
+    const int Xn = __shfl_sync(0xffffffffu, nb_l, d);
+    const Piece* v = reinterpret_cast<const Piece*>(in + (int64_t)Xn * nc) + l;
+    T r = T(0), q = T(0);
+    auto add = [&](const Piece& w, const Piece& x) {
+#pragma unroll
+      for (int e = 0; e < PER; e++) {
+        r = fma(w.v[e].r, x.v[e].r, fma(-w.v[e].i, x.v[e].i, r));
+        q = fma(w.v[e].r, x.v[e].i, fma(w.v[e].i, x.v[e].r, q));
+      }
+    };
+    if constexpr (NP > 0) {
+#pragma unroll
+      for (int p = 0; p < NP; p++) add(y[p * CA_LANES], v[p * CA_LANES]);
+    } else {
+      for (int p = 0; p + l < pieces; p += CA_LANES) add(y[p], v[p]);
+    }
+    sr = add_term(sr, r);
+    si = add_term(si, q);
+    y += ystep;
+  }
+#pragma unroll
+  for (int o = CA_LANES / 2; o > 0; o >>= 1) {
+    sr = sr + xor_lanes(sr, o);
+    si = si + xor_lanes(si, o);
+  }
+  if (l == 0 && i < nc) out[(int64_t)X * nc + i] = mk((T)sum_value(sr), (T)sum_value(si));
+}
+
+// The adjoint, out(X)_i = sum_d sum_j conj(Y_{-d}(X + d)_ji) in(X + d)_j, from the
+// blocks as they are stored (the solver keeps the adjoint stencil's own blocks
+// and uses k_coarse_apply). One warp per (coarse site, row): the lanes take the
+// 9 Nc products in turn and the warp sums them.
 template <typename T>
-__global__ void __launch_bounds__(MG_BLOCK) k_coarse_apply(cpx<T>* out, const cpx<T>* in, const cpx<T>* Y, MGGeom m,
-                                                           int dagger) {
+__global__ void __launch_bounds__(MG_BLOCK) k_coarse_apply_dag(cpx<T>* out, const cpx<T>* in, const cpx<T>* Y,
+                                                               MGGeom m) {
   const int64_t wid = ((int64_t)blockIdx.x * MG_BLOCK + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (wid >= m.Vc * m.nc) return;  // whole warps exit together
@@ -357,13 +476,8 @@ __global__ void __launch_bounds__(MG_BLOCK) k_coarse_apply(cpx<T>* out, const cp
     if (q >= total) continue;
     const int j = q - d * nc;
     const cpx<T> v = in[(int64_t)Xn * nc + j];
-    cpx<T> y;
-    if (!dagger) {
-      y = Y[(((int64_t)d * m.Vc + X) * nc + i) * nc + j];
-    } else {
-      const int dr = d == 0 ? 0 : (((d - 1) ^ 1) + 1);  // opposite direction
-      y = conj(Y[(((int64_t)dr * m.Vc + Xn) * nc + j) * nc + i]);
-    }
+    const int dr = d == 0 ? 0 : (((d - 1) ^ 1) + 1);  // opposite direction
+    const cpx<T> y = conj(Y[(((int64_t)dr * m.Vc + Xn) * nc + j) * nc + i]);
     const cpx<T> p = cmul(y, v);
     if (sizeof(T) == 8) {
       dr_ += (double)p.r;
@@ -653,8 +767,9 @@ template <typename F> static int dispatch_prec(int prec, F&& f) {
 
 static int restrict_(const MGGeom& m, int prec, void* coarse, const void* fine, const void* vecs, cudaStream_t s) {
   return dispatch_prec(prec, [&](auto P) {
-    k_restrict<decltype(P)::value><<<dim3((unsigned)m.Vc, (unsigned)m.nv), agg_threads(m), 0, s>>>(coarse, fine, vecs,
-                                                                                                 m);
+    constexpr int PR = decltype(P)::value;
+    if (m.b == 4) k_restrict<PR, 4><<<(unsigned)m.Vc, RS_BLOCK, 0, s>>>(coarse, fine, vecs, m);
+    else k_restrict<PR, 2><<<(unsigned)((m.Vc + 15) / 16), RS_BLOCK, 0, s>>>(coarse, fine, vecs, m);
     return after_launch("k_restrict");
   });
 }
@@ -665,18 +780,32 @@ static int prolong_(const MGGeom& m, int prec, void* fine, const void* coarse, c
     return after_launch("k_prolong");
   });
 }
+template <typename T>
+static void launch_coarse_apply(const MGGeom& m, void* out, const void* in, const void* Y, int dagger, cudaStream_t s) {
+  const int64_t warps = dagger ? m.Vc * m.nc : m.Vc * ((m.nc * CA_LANES + 31) / 32);
+  auto* o = static_cast<cpx<T>*>(out);
+  auto* i = static_cast<const cpx<T>*>(in);
+  auto* y = static_cast<const cpx<T>*>(Y);
+  if (dagger) k_coarse_apply_dag<T><<<n_grid(warps * 32), MG_BLOCK, 0, s>>>(o, i, y, m);
+  else {
+    const int pieces = m.nc * (int)sizeof(cpx<T>) / 16;
+    const unsigned grid = n_grid(warps * 32);
+    switch (pieces % CA_LANES ? 0 : pieces / CA_LANES) {
+      case 1: k_coarse_apply<T, 1><<<grid, MG_BLOCK, 0, s>>>(o, i, y, m); break;
+      case 2: k_coarse_apply<T, 2><<<grid, MG_BLOCK, 0, s>>>(o, i, y, m); break;
+      case 3: k_coarse_apply<T, 3><<<grid, MG_BLOCK, 0, s>>>(o, i, y, m); break;
+      case 4: k_coarse_apply<T, 4><<<grid, MG_BLOCK, 0, s>>>(o, i, y, m); break;
+      case 5: k_coarse_apply<T, 5><<<grid, MG_BLOCK, 0, s>>>(o, i, y, m); break;
+      case 6: k_coarse_apply<T, 6><<<grid, MG_BLOCK, 0, s>>>(o, i, y, m); break;
+      default: k_coarse_apply<T, 0><<<grid, MG_BLOCK, 0, s>>>(o, i, y, m);
+    }
+  }
+}
 static int coarse_apply_(const MGGeom& m, int prec, void* out, const void* in, const void* Y, int dagger,
                          cudaStream_t s) {
-  const unsigned grid = n_grid(m.Vc * m.nc * 32);
-  if (prec == LQCD_F64)
-    k_coarse_apply<double><<<grid, MG_BLOCK, 0, s>>>(static_cast<cpx<double>*>(out),
-                                                     static_cast<const cpx<double>*>(in),
-                                                     static_cast<const cpx<double>*>(Y), m, dagger);
-  else if (prec == LQCD_F32)
-    k_coarse_apply<float><<<grid, MG_BLOCK, 0, s>>>(static_cast<cpx<float>*>(out), static_cast<const cpx<float>*>(in),
-                                                    static_cast<const cpx<float>*>(Y), m, dagger);
-  else
-    return fail(LQCD_ERR_ARG, "multigrid: precision must be LQCD_F64 or LQCD_F32");
+  if (prec == LQCD_F64) launch_coarse_apply<double>(m, out, in, Y, dagger, s);
+  else if (prec == LQCD_F32) launch_coarse_apply<float>(m, out, in, Y, dagger, s);
+  else return fail(LQCD_ERR_ARG, "multigrid: precision must be LQCD_F64 or LQCD_F32");
   return after_launch("k_coarse_apply");
 }
 static int orthonormalize_(const MGGeom& m, void* vecs, cudaStream_t s) {
