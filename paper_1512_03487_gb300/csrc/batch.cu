@@ -104,11 +104,7 @@ __global__ void __launch_bounds__(TILE) batch_hop_kernel(const BatchArgs A) {
     const int64_t j = (t - s_t0[k]) * TILE + threadIdx.x;
     double v = 0.0;
     if (j < I.g.nsites) {
-      EpiCoef c;
-      c.a = I.c;
-      c.b = EPI == EPI_XPAY ? I.b : 1.0;
-      c.m5d = 0.0;
-      c.mf = 0.0;
+      const EpiCoef<T> c{(T)I.c, EPI == EPI_XPAY ? (T)I.b : T(1), T(0), T(0)};
       Spinor<T> res;
       hop_site<P, R, DAG, EPI>(I.g, A.use64 ? I.gauge64 : I.gauge_s, I.f[A.f_in],
                                A.f_x == BF_NONE ? nullptr : I.f[A.f_x], A.out_parity, j, c, res);

@@ -44,6 +44,8 @@ struct HopArgs {
   int m5_dagger;          // EPI_M5INV: apply the adjoint of M5op^-1
   double m5_a;            // EPI_M5INV: 1 / (5 - M5)
   double m5_den_inv;      // EPI_M5INV: 1 / (1 + mf (5 - M5)^-L_s)
+  float af, bf, m5df, mff, m5_af, m5_den_invf;  // the same rounded once on the host (set_float_coefs): a
+                          // conversion in the kernel is an FP64-pipe instruction per thread
   ReduceCtx red;          // |out|^2 per system (RED_NORM) or |r_s|^2 (RED_CG_UPDATE)
   const Control* gate;    // kernel returns at once when gate->active == 0
   // RED_CG_UPDATE: out = A p is not stored; instead x_s += alpha p and
@@ -55,6 +57,15 @@ struct HopArgs {
   int64_t upd_half_bytes;
   int64_t upd_rs_half_bytes;
 };
+
+inline void set_float_coefs(HopArgs& h) {
+  h.af = (float)h.a;
+  h.bf = (float)h.b;
+  h.m5df = (float)h.m5d;
+  h.mff = (float)h.mf;
+  h.m5_af = (float)h.m5_a;
+  h.m5_den_invf = (float)h.m5_den_inv;
+}
 
 // Reduction / epilogue modes of the hop kernel.
 enum HopReduce { RED_NONE = 0, RED_NORM = 1, RED_CG_UPDATE = 2 };
@@ -227,11 +238,11 @@ __device__ __forceinline__ void project_f16_words(const unsigned int (&w)[12], H
 template <int MU, int S>
 __device__ __forceinline__ float load_project_f16(const void* in, int64_t stride, int64_t idx, Half<float>& h) {
   const uint4* b = reinterpret_cast<const uint4*>(in);
-  const float nrm = __ldg(SpinorIO<LQCD_F16>::norm_ptr(in, stride) + idx);
+  const float nrm = SpinorIO<LQCD_F16>::norm_ptr(in, stride)[idx];
   unsigned int w[12];
 #pragma unroll
   for (int c = 0; c < 3; c++) {
-    const uint4 v = __ldg(b + c * stride + idx);
+    const uint4 v = b[c * stride + idx];
     w[4 * c] = v.x;
     w[4 * c + 1] = v.y;
     w[4 * c + 2] = v.z;
@@ -338,9 +349,25 @@ __device__ __forceinline__ void add_chiral(Spinor<T>& out, const Spinor<T>& xs, 
 // M5 out = M5op(x) + b H in with M5op diagonal m5d and corner mf. (Loading the
 // xpay operand before the hop, as the accumulator's start, made the bench step
 // 1.8 % slower with FP16 storage: the operand is read at the end.)
-struct EpiCoef {
-  double a, b, m5d, mf;
+template <typename T> struct EpiCoef {
+  T a, b, m5d, mf;
 };
+template <typename T> __device__ __forceinline__ EpiCoef<T> epi_coef(const HopArgs& A) {
+  return EpiCoef<T>{(T)A.a, (T)A.b, (T)A.m5d, (T)A.mf};
+}
+template <> __device__ __forceinline__ EpiCoef<float> epi_coef<float>(const HopArgs& A) {
+  return EpiCoef<float>{A.af, A.bf, A.m5df, A.mff};
+}
+// The M5op^-1 scan's coefficients a, mf, 1 / (1 + mf a^L_s)
+template <typename T> struct M5Coef {
+  T a, mf, den_inv;
+};
+template <typename T> __device__ __forceinline__ M5Coef<T> m5_coef(const HopArgs& A) {
+  return M5Coef<T>{(T)A.m5_a, (T)A.mf, (T)A.m5_den_inv};
+}
+template <> __device__ __forceinline__ M5Coef<float> m5_coef<float>(const HopArgs& A) {
+  return M5Coef<float>{A.m5_af, A.mff, A.m5_den_invf};
+}
 
 // Both hops along mu with spin-paired packed arithmetic (hop_pair.cuh): the
 // projection and the link as in hop_dir, the products and the accumulation on
@@ -436,20 +463,21 @@ __device__ __forceinline__ void hop_acc(const Geom& g, const void* gauge, const 
 
 // The epilogue at output site j of the hop result acc = H in (see EpiCoef).
 template <int P, bool DAG, int EPI>
-__device__ __forceinline__ void hop_epilogue(const Geom& g, const void* xb, int64_t j, const EpiCoef& c,
+__device__ __forceinline__ void hop_epilogue(const Geom& g, const void* xb, int64_t j,
+                                             const EpiCoef<typename PrecTraits<P>::real>& c,
                                              const Spinor<typename PrecTraits<P>::real>& acc,
                                              Spinor<typename PrecTraits<P>::real>& res) {
   using T = typename PrecTraits<P>::real;
   using IO = SpinorIO<P>;
   const int64_t n5 = g.n5;
-  const T b = (T)c.b;
+  const T b = c.b;
   if (EPI == EPI_PLAIN || EPI == EPI_M5INV) {
 #pragma unroll
     for (int k = 0; k < 12; k++) res.v[k] = b * acc.v[k];
   } else if (EPI == EPI_XPAY) {
     Spinor<T> xv;
     IO::load(xb, g.sstride, j, xv);
-    const T a = (T)c.a;
+    const T a = c.a;
 #pragma unroll
     for (int k = 0; k < 12; k++) res.v[k] = mk(fma(a, xv.v[k].r, b * acc.v[k].r), fma(a, xv.v[k].i, b * acc.v[k].i));
   } else {
@@ -457,14 +485,14 @@ __device__ __forceinline__ void hop_epilogue(const Geom& g, const void* xb, int6
     const int64_t i5 = n5 == 1 ? 0 : j - (int64_t)fdiv((uint32_t)j, g.fn5) * n5;
     Spinor<T> xv;
     IO::load(xb, g.sstride, j, xv);
-    const T d = (T)c.m5d;
+    const T d = c.m5d;
 #pragma unroll
     for (int k = 0; k < 12; k++) res.v[k] = mk(fma(d, xv.v[k].r, b * acc.v[k].r), fma(d, xv.v[k].i, b * acc.v[k].i));
     const bool top = i5 + 1 == n5, bottom = i5 == 0;
     const int64_t jp = top ? j - (n5 - 1) : j + 1;
     const int64_t jm = bottom ? j + (n5 - 1) : j - 1;
-    const T cp = top ? (T)c.mf : T(-1);
-    const T cm = bottom ? (T)c.mf : T(-1);
+    const T cp = top ? c.mf : T(-1);
+    const T cm = bottom ? c.mf : T(-1);
     Spinor<T> xp, xm;
     IO::load(xb, g.sstride, jp, xp);
     IO::load(xb, g.sstride, jm, xm);
@@ -481,7 +509,7 @@ __device__ __forceinline__ void hop_epilogue(const Geom& g, const void* xb, int6
 // The result at output site j (= cb * n5 + i5) of checkerboard `parity`.
 template <int P, int R, bool DAG, int EPI, bool GP = false, bool SP = false, bool AS = false, int BLOCK = 128>
 __device__ __forceinline__ void hop_site(const Geom& g, const void* gauge, const void* in, const void* xb,
-                                         int parity, int64_t j, const EpiCoef& c,
+                                         int parity, int64_t j, const EpiCoef<typename PrecTraits<P>::real>& c,
                                          Spinor<typename PrecTraits<P>::real>& res,
                                          const Link<typename PrecTraits<P>::real>* sl = nullptr,
                                          unsigned char* ring = nullptr) {
@@ -552,6 +580,7 @@ template <int P, int R, bool DAG, int EPI, int RED, int BLOCK, bool GP, int SPT,
 __device__ __forceinline__ void hop_body(const HopArgs& A) {
   using T = typename PrecTraits<P>::real;
   static_assert(SPT == 1 || (SPT == 2 && P != LQCD_F64 && !GP), "two sites per thread: FP32 / FP16, no G-parity");
+  overlap_launch();
   if (gate_closed(A.gate)) return;
   int parity = A.out_parity;
   int blk = blockIdx.x;
@@ -562,7 +591,7 @@ __device__ __forceinline__ void hop_body(const HopArgs& A) {
   const char* in = static_cast<const char*>(A.in) + (A.full ? (1 - parity) * A.half_bytes : 0);
   char* out = static_cast<char*>(A.out) + (A.full ? parity * A.half_bytes : 0);
   const char* xb = A.x ? static_cast<const char*>(A.x) + (A.full ? parity * A.half_bytes : 0) : nullptr;
-  const EpiCoef c{A.a, A.b, A.m5d, A.mf};
+  const EpiCoef<T> c = epi_coef<T>(A);
   const int64_t first = (int64_t)blk * (BLOCK * SPT);
   if constexpr (SPT == 1) {
     const int64_t j = first + threadIdx.x;
@@ -593,8 +622,8 @@ __device__ __forceinline__ void hop_body(const HopArgs& A) {
       if (live) hop_site<P, R, DAG, EPI, GP, SP, AS, BLOCK>(A.g, A.gauge, in, xb, parity, j, c, res, sl, ring);
       else zero(res);
       const int Ls = A.g.n5;
-      m5inv_lanes(res, (int)(threadIdx.x & (unsigned)(Ls - 1)), Ls, A.m5_dagger != 0, (T)A.m5_a, (T)A.mf,
-                  (T)A.m5_den_inv);
+      const M5Coef<T> mc = m5_coef<T>(A);
+      m5inv_lanes(res, (int)(threadIdx.x & (unsigned)(Ls - 1)), Ls, A.m5_dagger != 0, mc.a, mc.mf, mc.den_inv);
       if (live) SpinorIO<P>::store(out, A.g.sstride, j, res);
       return;
     }
@@ -642,8 +671,8 @@ __device__ __forceinline__ void hop_body(const HopArgs& A) {
         Spinor<T> res;
         if (live[s]) hop_epilogue<P, DAG, EPI>(A.g, xb, j[s], c, acc[s], res);
         else zero(res);
-        m5inv_lanes(res, (int)(threadIdx.x & (unsigned)(Ls - 1)), Ls, A.m5_dagger != 0, (T)A.m5_a, (T)A.mf,
-                    (T)A.m5_den_inv);
+        const M5Coef<T> mc = m5_coef<T>(A);
+        m5inv_lanes(res, (int)(threadIdx.x & (unsigned)(Ls - 1)), Ls, A.m5_dagger != 0, mc.a, mc.mf, mc.den_inv);
         if (live[s]) SpinorIO<P>::store(out, A.g.sstride, j[s], res);
       }
     } else {

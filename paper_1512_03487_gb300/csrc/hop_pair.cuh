@@ -65,8 +65,8 @@ template <> struct PairSpinorIO<LQCD_F32> {
     const float4* b = reinterpret_cast<const float4*>(base);
 #pragma unroll
     for (int c = 0; c < 6; c++) {
-      const float4 wa = __ldg(b + c * stride + ja);
-      const float4 wb = __ldg(b + c * stride + jb);
+      const float4 wa = b[c * stride + ja];
+      const float4 wb = b[c * stride + jb];
       s.v[2 * c] = pmk(make_float2(wa.x, wb.x), make_float2(wa.y, wb.y));
       s.v[2 * c + 1] = pmk(make_float2(wa.z, wb.z), make_float2(wa.w, wb.w));
     }
@@ -79,11 +79,11 @@ template <> struct PairSpinorIO<LQCD_F16> {
                                               float2& nrm) {
     const uint4* b = reinterpret_cast<const uint4*>(base);
     const float* np = reinterpret_cast<const float*>(reinterpret_cast<const char*>(base) + 48 * stride);
-    nrm = make_float2(__ldg(np + ja), __ldg(np + jb));
+    nrm = make_float2(np[ja], np[jb]);
 #pragma unroll
     for (int c = 0; c < 3; c++) {
-      const uint4 wa = __ldg(b + c * stride + ja);
-      const uint4 wb = __ldg(b + c * stride + jb);
+      const uint4 wa = b[c * stride + ja];
+      const uint4 wb = b[c * stride + jb];
       const unsigned int a4[4] = {wa.x, wa.y, wa.z, wa.w};
       const unsigned int b4[4] = {wb.x, wb.y, wb.z, wb.w};
 #pragma unroll
@@ -123,7 +123,7 @@ template <> struct PairLinkIO<LQCD_F32, 12> {
     const float4* bb = reinterpret_cast<const float4*>(g) + (int64_t)blk_b * 3 * gs + cb_b;
 #pragma unroll
     for (int c = 0; c < 3; c++) {
-      const float4 wa = __ldg(ba + c * gs), wb = __ldg(bb + c * gs);
+      const float4 wa = ba[c * gs], wb = bb[c * gs];
       u.v[2 * c] = pmk(make_float2(wa.x, wb.x), make_float2(wa.y, wb.y));
       u.v[2 * c + 1] = pmk(make_float2(wa.z, wb.z), make_float2(wa.w, wb.w));
     }
@@ -137,7 +137,7 @@ template <> struct PairLinkIO<LQCD_F32, 18> {
     const float2* bb = reinterpret_cast<const float2*>(g) + (int64_t)blk_b * 9 * gs + cb_b;
 #pragma unroll
     for (int c = 0; c < 9; c++) {
-      const float2 wa = __ldg(ba + c * gs), wb = __ldg(bb + c * gs);
+      const float2 wa = ba[c * gs], wb = bb[c * gs];
       u.v[c] = pmk(make_float2(wa.x, wb.x), make_float2(wa.y, wb.y));
     }
   }
@@ -149,7 +149,7 @@ template <> struct PairLinkIO<LQCD_F16, 12> {
     const uint2* bb = reinterpret_cast<const uint2*>(g) + (int64_t)blk_b * 3 * gs + cb_b;
 #pragma unroll
     for (int c = 0; c < 3; c++) {
-      const uint2 wa = __ldg(ba + c * gs), wb = __ldg(bb + c * gs);
+      const uint2 wa = ba[c * gs], wb = bb[c * gs];
       u.v[2 * c] = pmk(h2lo_hi(wa.x, wb.x, false), h2lo_hi(wa.x, wb.x, true));
       u.v[2 * c + 1] = pmk(h2lo_hi(wa.y, wb.y, false), h2lo_hi(wa.y, wb.y, true));
     }
@@ -163,7 +163,7 @@ template <> struct PairLinkIO<LQCD_F16, 18> {
     const unsigned int* bb = reinterpret_cast<const unsigned int*>(g) + (int64_t)blk_b * 9 * gs + cb_b;
 #pragma unroll
     for (int c = 0; c < 9; c++) {
-      const unsigned int wa = __ldg(ba + c * gs), wb = __ldg(bb + c * gs);
+      const unsigned int wa = ba[c * gs], wb = bb[c * gs];
       u.v[c] = pmk(h2lo_hi(wa, wb, false), h2lo_hi(wa, wb, true));
     }
   }

@@ -27,6 +27,39 @@ int after_launch(const char* what);
 
 inline int64_t round_up(int64_t a, int64_t b) { return (a + b - 1) / b * b; }
 
+// Launches kernel so that it may start while the kernel before it on the stream still
+// runs (programmatic dependent launch): its blocks take the SMs that the other's last
+// blocks leave idle and do their index arithmetic there. The kernel calls
+// overlap_launch() before it touches memory. A predecessor that does not take part
+// is waited for as usual. Back to back on one stream it gains 7-8 % at 24^3 x 48 and
+// below (FP16 M^dag M 110 -> 102 us, 8^4 FP32 24.6 -> 22.8 us); in the bodies of the
+// solver's conditional graph it loses 7 % (158 -> 169 us an iteration), so a captured
+// launch is an ordinary one.
+template <typename Arg>
+inline cudaError_t launch_overlapped(void (*kernel)(Arg), unsigned grid, unsigned block, cudaStream_t s, const Arg& arg) {
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  const cudaError_t e = cudaStreamIsCapturing(s, &capture);
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = capture == cudaStreamCaptureStatusNone;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, arg);
+}
+// Lets the next kernel on the stream start and waits until the ones before have
+// finished and their writes are visible. Every thread of every block calls it, also
+// one that returns at once: a kernel that ended without waiting would release its
+// successor while its predecessor still runs.
+__device__ __forceinline__ void overlap_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ------------------------------------------------------------------ geometry
 // Division of n < 2^31 by a runtime constant d >= 1 with one multiply-high,
 // an add and a shift (Granlund and Montgomery, "Division by invariant
@@ -138,6 +171,9 @@ struct CFieldPtr {
   int64_t stride;
 };
 
+// Spinors are read with ordinary loads, not through the read-only path: a kernel that
+// starts before its predecessor has finished (overlap_launch) may read them only after
+// it has waited, and only an ordinary load is ordered behind that wait.
 template <int P> struct SpinorIO;
 
 template <> struct SpinorIO<LQCD_F64> {
@@ -146,7 +182,7 @@ template <> struct SpinorIO<LQCD_F64> {
     const double2* b = reinterpret_cast<const double2*>(base);
 #pragma unroll
     for (int c = 0; c < 12; c++) {
-      double2 w = __ldg(b + c * stride + j);
+      double2 w = b[c * stride + j];
       s.v[c] = mk(w.x, w.y);
     }
   }
@@ -163,7 +199,7 @@ template <> struct SpinorIO<LQCD_F32> {
     const float4* b = reinterpret_cast<const float4*>(base);
 #pragma unroll
     for (int c = 0; c < 6; c++) {
-      float4 w = __ldg(b + c * stride + j);
+      float4 w = b[c * stride + j];
       s.v[2 * c] = mk(w.x, w.y);
       s.v[2 * c + 1] = mk(w.z, w.w);
     }
@@ -184,7 +220,7 @@ template <> struct SpinorIO<LQCD_F64_DF> {
     const double2* b = reinterpret_cast<const double2*>(base);
 #pragma unroll
     for (int c = 0; c < 12; c++) {
-      const double2 w = __ldg(b + c * stride + j);
+      const double2 w = b[c * stride + j];
       s.v[c] = mk(df_split(w.x), df_split(w.y));
     }
   }
@@ -203,10 +239,10 @@ template <> struct SpinorIO<LQCD_F16> {
   }
   static __device__ __forceinline__ void load(const void* base, int64_t stride, int64_t j, Spinor<T>& s) {
     const uint4* b = reinterpret_cast<const uint4*>(base);
-    float nrm = __ldg(norm_ptr(base, stride) + j);
+    float nrm = norm_ptr(base, stride)[j];
 #pragma unroll
     for (int c = 0; c < 3; c++) {
-      uint4 w = __ldg(b + c * stride + j);
+      uint4 w = b[c * stride + j];
       unsigned int words[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
       for (int q = 0; q < 4; q++) {
@@ -221,10 +257,10 @@ template <> struct SpinorIO<LQCD_F16> {
   static __device__ __forceinline__ void load_unscaled(const void* base, int64_t stride, int64_t j, Spinor<T>& s,
                                                        float& nrm) {
     const uint4* b = reinterpret_cast<const uint4*>(base);
-    nrm = __ldg(norm_ptr(base, stride) + j);
+    nrm = norm_ptr(base, stride)[j];
 #pragma unroll
     for (int c = 0; c < 3; c++) {
-      uint4 w = __ldg(b + c * stride + j);
+      uint4 w = b[c * stride + j];
       unsigned int words[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
       for (int q = 0; q < 4; q++) {
@@ -255,7 +291,7 @@ template <> struct SpinorIO<LQCD_F16> {
 };
 
 // ------------------------------------------------------------------ link I/O
-// Gauge block (parity, mu) starts at chunk (parity * 4 + mu) * NCHUNK.
+// Gauge block (parity, mu) starts at chunk (parity * 4 + mu) * NCHUNK. Ordinary loads, as for spinors.
 template <int P, int R> struct LinkIO;
 
 // conj(a b - c d) as two chains of a multiply and three fused multiply-adds
@@ -284,7 +320,7 @@ template <> struct LinkIO<LQCD_F64, 18> {
   static __device__ __forceinline__ void load(const void* g, int64_t gs, int blk, int64_t cb, Link<T>& u) {
     const double2* b = reinterpret_cast<const double2*>(g) + (int64_t)blk * NCHUNK * gs + cb;
 #pragma unroll
-    for (int c = 0; c < 9; c++) { double2 w = __ldg(b + c * gs); u.v[c] = mk(w.x, w.y); }
+    for (int c = 0; c < 9; c++) { double2 w = b[c * gs]; u.v[c] = mk(w.x, w.y); }
   }
 };
 template <> struct LinkIO<LQCD_F64, 12> {
@@ -293,7 +329,7 @@ template <> struct LinkIO<LQCD_F64, 12> {
   static __device__ __forceinline__ void load(const void* g, int64_t gs, int blk, int64_t cb, Link<T>& u) {
     const double2* b = reinterpret_cast<const double2*>(g) + (int64_t)blk * NCHUNK * gs + cb;
 #pragma unroll
-    for (int c = 0; c < 6; c++) { double2 w = __ldg(b + c * gs); u.v[c] = mk(w.x, w.y); }
+    for (int c = 0; c < 6; c++) { double2 w = b[c * gs]; u.v[c] = mk(w.x, w.y); }
     rebuild_row2(u);
   }
 };
@@ -303,7 +339,7 @@ template <> struct LinkIO<LQCD_F64_DF, 18> {
   static __device__ __forceinline__ void load(const void* g, int64_t gs, int blk, int64_t cb, Link<T>& u) {
     const double2* b = reinterpret_cast<const double2*>(g) + (int64_t)blk * NCHUNK * gs + cb;
 #pragma unroll
-    for (int c = 0; c < 9; c++) { double2 w = __ldg(b + c * gs); u.v[c] = mk(df_split(w.x), df_split(w.y)); }
+    for (int c = 0; c < 9; c++) { double2 w = b[c * gs]; u.v[c] = mk(df_split(w.x), df_split(w.y)); }
   }
 };
 template <> struct LinkIO<LQCD_F64_DF, 12> {
@@ -312,7 +348,7 @@ template <> struct LinkIO<LQCD_F64_DF, 12> {
   static __device__ __forceinline__ void load(const void* g, int64_t gs, int blk, int64_t cb, Link<T>& u) {
     const double2* b = reinterpret_cast<const double2*>(g) + (int64_t)blk * NCHUNK * gs + cb;
 #pragma unroll
-    for (int c = 0; c < 6; c++) { double2 w = __ldg(b + c * gs); u.v[c] = mk(df_split(w.x), df_split(w.y)); }
+    for (int c = 0; c < 6; c++) { double2 w = b[c * gs]; u.v[c] = mk(df_split(w.x), df_split(w.y)); }
     rebuild_row2(u);
   }
 };
@@ -322,7 +358,7 @@ template <> struct LinkIO<LQCD_F32, 18> {
   static __device__ __forceinline__ void load(const void* g, int64_t gs, int blk, int64_t cb, Link<T>& u) {
     const float2* b = reinterpret_cast<const float2*>(g) + (int64_t)blk * NCHUNK * gs + cb;
 #pragma unroll
-    for (int c = 0; c < 9; c++) { float2 w = __ldg(b + c * gs); u.v[c] = mk(w.x, w.y); }
+    for (int c = 0; c < 9; c++) { float2 w = b[c * gs]; u.v[c] = mk(w.x, w.y); }
   }
 };
 template <> struct LinkIO<LQCD_F32, 12> {
@@ -332,7 +368,7 @@ template <> struct LinkIO<LQCD_F32, 12> {
     const float4* b = reinterpret_cast<const float4*>(g) + (int64_t)blk * NCHUNK * gs + cb;
 #pragma unroll
     for (int c = 0; c < 3; c++) {
-      float4 w = __ldg(b + c * gs);
+      float4 w = b[c * gs];
       u.v[2 * c] = mk(w.x, w.y);
       u.v[2 * c + 1] = mk(w.z, w.w);
     }
@@ -346,7 +382,7 @@ template <> struct LinkIO<LQCD_F16, 18> {
     const unsigned int* b = reinterpret_cast<const unsigned int*>(g) + (int64_t)blk * NCHUNK * gs + cb;
 #pragma unroll
     for (int c = 0; c < 9; c++) {
-      unsigned int w = __ldg(b + c * gs);
+      unsigned int w = b[c * gs];
       float2 f = __half22float2(*reinterpret_cast<__half2*>(&w));
       u.v[c] = mk(f.x, f.y);
     }
@@ -359,7 +395,7 @@ template <> struct LinkIO<LQCD_F16, 12> {
     const uint2* b = reinterpret_cast<const uint2*>(g) + (int64_t)blk * NCHUNK * gs + cb;
 #pragma unroll
     for (int c = 0; c < 3; c++) {
-      uint2 w = __ldg(b + c * gs);
+      uint2 w = b[c * gs];
       float2 f0 = __half22float2(*reinterpret_cast<__half2*>(&w.x));
       float2 f1 = __half22float2(*reinterpret_cast<__half2*>(&w.y));
       u.v[2 * c] = mk(f0.x, f0.y);
