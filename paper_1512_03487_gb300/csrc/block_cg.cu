@@ -203,8 +203,8 @@ __device__ void block_finalize(const BlockArgs& a, const cpx<double>* M, cpx<dou
           c.active = 0;
         } else if (reason || at_cap) {
           c.reason |= reason;
+          c.active = 0;  // pause: the kernels queued behind return at once
           if (a.cond) cudaGraphSetConditional(a.h_rel, 1);
-          else c.active = 0;
         } else {
           go = 1;
         }

@@ -506,7 +506,7 @@ struct ReduceCtx {
                           // of result[s] (an even-odd solve: the full system's source, so that tol applies to
                           // ||b - D x|| / ||b||, whose even rows are b_hat - M_hat x_e and odd rows vanish)
   int maxiter;            // FIN_UPDATE: request a final FP64 residual once this many iterations ran
-  int cond;               // FIN_UPDATE: 1 = set h_rel / h_mid (device-driven graph), 0 = pause for the host
+  int cond;               // FIN_UPDATE: 1 = set h_rel / h_mid as well as pausing (device-driven graph)
   cudaGraphConditionalHandle h_rel;  // IF node running the reliable update (when cond)
   cudaGraphConditionalHandle h_mid;  // IF node running the FP32-arithmetic replacement (when cond)
 };
@@ -557,8 +557,8 @@ __device__ inline void finalize_totals(const ReduceCtx& rc, const double* totals
         // iteration cap, where the true residual must be known) or, failing
         // those, the FP32-arithmetic replacement: beta waits for it.
         rc.ctrl->reason |= rel_due ? (reason & ~REASON_MID) : REASON_MID;
-        if (rc.cond) cudaGraphSetConditional(rel_due ? rc.h_rel : rc.h_mid, 1);  // run that branch now
-        else rc.ctrl->active = 0;                                                  // pause for the host
+        rc.ctrl->active = 0;  // pause: the kernels queued behind return at once
+        if (rc.cond) cudaGraphSetConditional(rel_due ? rc.h_rel : rc.h_mid, 1);  // the graph's branch, else the host
       } else {
         for (int s = 0; s < nsys; s++) {
           SysState& st = rc.sys[s];

@@ -1,5 +1,8 @@
-"""Launches that start while their predecessor runs: chains without host
-synchronisation give the bits of the same chain synchronised after every call."""
+"""Launches that start while their predecessor runs, and several iterations per body of
+the solver's graph: chains without host synchronisation give the bits of the same
+chain synchronised after every call, and a solve's iterations, updates and solution
+do not depend on how many iterations a graph body holds."""
+import numpy as np
 import pytest
 
 from synthetic import gauge_field, gaussian_spinor
@@ -58,3 +61,49 @@ def test_chained_operators_without_synchronisation(L, dims, prec, recon, stream)
     expect = chain(True)
     for _ in range(5):
         assert torch.equal(chain(False), expect)
+
+
+@pytest.mark.parametrize("sloppy,mid", [(0, 0.0), (1, 0.0), (2, 0.01)])
+def test_solve_does_not_depend_on_the_iterations_per_graph_body(L, sloppy, mid):
+    F = L.fields
+    dims, m = (4, 4, 4, 8), 0.05
+    lat = L.lattice(dims, bc=BC)
+    op = L.operator(mass=m)
+    U, b = gauge_field(dims, "haar", 2311), gaussian_spinor(dims, 2312, lead=(1,))
+    g64 = F.gauge_to_device(U, lat, 0, 18)
+    gs = F.gauge_to_device(U, lat, sloppy, 12) if sloppy else g64
+    bd = F.spinor_to_device(b, lat, 0, L.LQCD_FULL)
+    seen = []
+    for check in (1, 2, 3, 7, 8, 11, 12, 64):  # 1, 2, 3, 7, 8, 1, 6, 8 iterations per body
+        prm = L.solver_params(tol=1e-10, maxiter=500, sloppy_prec=sloppy, sloppy_recon=12, delta=1e-3, delta_mid=mid,
+                              check_interval=check)
+        ws = F.empty(L.lqcd_eo_solve_workspace_bytes(lat, op, prm))
+        x = F.empty(L.lqcd_spinor_bytes(lat, 0, L.LQCD_FULL))
+        i = L.lqcd_eo_solve(x, bd, g64, gs, lat, op, prm, ws)
+        seen.append((i.iterations, i.reliable_updates, i.residual_replacements, x.clone()))
+    for s in seen[1:]:
+        assert s[:3] == seen[0][:3]
+        assert torch.equal(s[3], seen[0][3])
+
+
+@pytest.mark.parametrize("maxiter", [1, 5, 8, 9])
+def test_iteration_cap_inside_a_body(L, maxiter):
+    """The cap ends the solve at exactly maxiter iterations, with the FP64 residual known."""
+    F = L.fields
+    dims = (4, 4, 4, 8)
+    lat = L.lattice(dims, bc=BC)
+    op = L.operator(mass=0.05)
+    U, b = gauge_field(dims, "haar", 2321), gaussian_spinor(dims, 2322, lead=(1,))
+    g64, g32 = F.gauge_to_device(U, lat, 0, 18), F.gauge_to_device(U, lat, 1, 12)
+    bd = F.spinor_to_device(b, lat, 0, L.LQCD_FULL)
+    x = F.empty(L.lqcd_spinor_bytes(lat, 0, L.LQCD_FULL))
+    res = []
+    for check, graph in ((64, 1), (1, 1), (1, 0)):
+        prm = L.solver_params(tol=1e-12, maxiter=maxiter, sloppy_prec=1, sloppy_recon=12, delta=0.0,
+                              check_interval=check, use_graph=graph)
+        ws = F.empty(L.lqcd_eo_solve_workspace_bytes(lat, op, prm))
+        i = L.lqcd_eo_solve(x, bd, g64, g32, lat, op, prm, ws, raise_on_error=False)
+        assert i.iterations == maxiter and i.status != 0
+        res.append(i.true_rel_residual)
+    assert np.isfinite(res).all() and res[0] == res[1]
+    assert res[0] == pytest.approx(res[2], rel=1e-6)  # the host-driven path: the same kernels
