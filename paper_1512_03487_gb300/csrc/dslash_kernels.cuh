@@ -283,13 +283,10 @@ template <typename T> __device__ __forceinline__ void conj_link(Link<T>& u) {
 // (forward, f = 0 / 1) or -1 / +1 (backward) instead of the boundary phase,
 // and the link is conjugated when its owner -- the site for the forward hop,
 // the neighbour (flavour f') for the backward hop -- is flavour 1.
-// sl: this 4D site's eight links staged in shared memory (forward link of mu
-// at 2 mu, the backward hop's link at 2 mu + 1), or null to load them here.
 template <int MU, int P, int R, bool DAG, bool GP = false>
 __device__ __forceinline__ void hop_dir(Spinor<typename PrecTraits<P>::real>& acc, const Geom& g,
                                         const void* gauge, const Coord& x, int64_t cb, int64_t i5,
-                                        int parity, const void* in,
-                                        const Link<typename PrecTraits<P>::real>* sl = nullptr) {
+                                        int parity, const void* in) {
   using T = typename PrecTraits<P>::real;
   constexpr int SF = DAG ? +1 : -1;  // forward hop carries (1 + SF gamma_mu)
   const int64_t n5 = g.n5;
@@ -306,8 +303,7 @@ __device__ __forceinline__ void hop_dir(Spinor<typename PrecTraits<P>::real>& ac
     Half<T> h;
     const T f = sgn * load_project<P, MU, SF>(in, g, nb * n5 + f_nb, wrap, h);
     Link<T> u;
-    if (sl) u = sl[2 * MU];
-    else LinkIO<P, R>::load(gauge, g.gstride, parity * 4 + MU, cb, u);
+    LinkIO<P, R>::load(gauge, g.gstride, parity * 4 + MU, cb, u);
     if (GP && i5 == 1) conj_link(u);
     Half<T> w;
     link_mul(u, h, w);
@@ -326,8 +322,7 @@ __device__ __forceinline__ void hop_dir(Spinor<typename PrecTraits<P>::real>& ac
     Half<T> h;
     const T f = sgn * load_project<P, MU, -SF>(in, g, nb * n5 + f_nb, wrap, h);
     Link<T> u;
-    if (sl) u = sl[2 * MU + 1];
-    else LinkIO<P, R>::load(gauge, g.gstride, (1 - parity) * 4 + MU, nb, u);
+    LinkIO<P, R>::load(gauge, g.gstride, (1 - parity) * 4 + MU, nb, u);
     if (GP && f_nb == 1) conj_link(u);
     Half<T> w;
     link_mul_dag(u, h, w);
@@ -374,7 +369,7 @@ template <> __device__ __forceinline__ M5Coef<float> m5_coef<float>(const HopArg
 // (spin 0, spin 1) pairs. FP32 / FP16 storage, no G-parity.
 template <int MU, int P, int R, bool DAG>
 __device__ __forceinline__ void hop_dir_sp(SPAcc& acc, const Geom& g, const void* gauge, const Coord& x, int64_t cb,
-                                           int64_t i5, int parity, const void* in, const Link<float>* sl) {
+                                           int64_t i5, int parity, const void* in) {
   constexpr int SF = DAG ? +1 : -1;
   const int64_t n5 = g.n5;
 #pragma unroll
@@ -392,13 +387,11 @@ __device__ __forceinline__ void hop_dir_sp(SPAcc& acc, const Geom& g, const void
     }
     Link<float> u;
     if (dir == 0) {
-      if (sl) u = sl[2 * MU];
-      else LinkIO<P, R>::load(gauge, g.gstride, parity * 4 + MU, cb, u);
+      LinkIO<P, R>::load(gauge, g.gstride, parity * 4 + MU, cb, u);
       link_mul_sp<false>(u, h, w);
       accumulate_sp<MU, SF>(acc, w, f);
     } else {
-      if (sl) u = sl[2 * MU + 1];
-      else LinkIO<P, R>::load(gauge, g.gstride, (1 - parity) * 4 + MU, nb, u);
+      LinkIO<P, R>::load(gauge, g.gstride, (1 - parity) * 4 + MU, nb, u);
       link_mul_sp<true>(u, h, w);
       accumulate_sp<MU, -SF>(acc, w, f);
     }
@@ -416,9 +409,7 @@ namespace lqcd {
 // data streamed through the shared-memory ring `ring` (hop_async.cuh).
 template <int P, int R, bool DAG, bool GP = false, bool SP = false, bool AS = false, int BLOCK = 128>
 __device__ __forceinline__ void hop_acc(const Geom& g, const void* gauge, const void* in, int parity, int64_t j,
-                                        Spinor<typename PrecTraits<P>::real>& acc,
-                                        const Link<typename PrecTraits<P>::real>* sl = nullptr,
-                                        unsigned char* ring = nullptr) {
+                                        Spinor<typename PrecTraits<P>::real>& acc, unsigned char* ring = nullptr) {
   if constexpr (P == LQCD_F64_DF) {
     hop_acc_df<R, DAG, AS, BLOCK>(g, gauge, in, parity, j, acc, ring);
     return;
@@ -439,26 +430,19 @@ __device__ __forceinline__ void hop_acc(const Geom& g, const void* gauge, const 
   if constexpr (SP) {
     static_assert(P == LQCD_F32 || P == LQCD_F16, "spin-paired hop: FP32 / FP16 storage");
     SPAcc a;
-#pragma unroll
-    for (int c = 0; c < 3; c++) a.ur[c] = a.ui[c] = a.lr[c] = a.li[c] = make_float2(0.f, 0.f);
-    hop_dir_sp<0, P, R, DAG>(a, g, gauge, x, cb, i5, parity, in, sl);
-    hop_dir_sp<1, P, R, DAG>(a, g, gauge, x, cb, i5, parity, in, sl);
-    hop_dir_sp<2, P, R, DAG>(a, g, gauge, x, cb, i5, parity, in, sl);
-    hop_dir_sp<3, P, R, DAG>(a, g, gauge, x, cb, i5, parity, in, sl);
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-      acc.v[c] = mk(a.ur[c].x, a.ui[c].x);
-      acc.v[3 + c] = mk(a.ur[c].y, a.ui[c].y);
-      acc.v[6 + c] = mk(a.lr[c].x, a.li[c].x);
-      acc.v[9 + c] = mk(a.lr[c].y, a.li[c].y);
-    }
+    sp_zero(a);
+    hop_dir_sp<0, P, R, DAG>(a, g, gauge, x, cb, i5, parity, in);
+    hop_dir_sp<1, P, R, DAG>(a, g, gauge, x, cb, i5, parity, in);
+    hop_dir_sp<2, P, R, DAG>(a, g, gauge, x, cb, i5, parity, in);
+    hop_dir_sp<3, P, R, DAG>(a, g, gauge, x, cb, i5, parity, in);
+    sp_unpack(a, acc);
     return;
   }
   zero(acc);
-  hop_dir<0, P, R, DAG, GP>(acc, g, gauge, x, cb, i5, parity, in, sl);
-  hop_dir<1, P, R, DAG, GP>(acc, g, gauge, x, cb, i5, parity, in, sl);
-  hop_dir<2, P, R, DAG, GP>(acc, g, gauge, x, cb, i5, parity, in, sl);
-  hop_dir<3, P, R, DAG, GP>(acc, g, gauge, x, cb, i5, parity, in, sl);
+  hop_dir<0, P, R, DAG, GP>(acc, g, gauge, x, cb, i5, parity, in);
+  hop_dir<1, P, R, DAG, GP>(acc, g, gauge, x, cb, i5, parity, in);
+  hop_dir<2, P, R, DAG, GP>(acc, g, gauge, x, cb, i5, parity, in);
+  hop_dir<3, P, R, DAG, GP>(acc, g, gauge, x, cb, i5, parity, in);
 }
 
 // The epilogue at output site j of the hop result acc = H in (see EpiCoef).
@@ -510,11 +494,9 @@ __device__ __forceinline__ void hop_epilogue(const Geom& g, const void* xb, int6
 template <int P, int R, bool DAG, int EPI, bool GP = false, bool SP = false, bool AS = false, int BLOCK = 128>
 __device__ __forceinline__ void hop_site(const Geom& g, const void* gauge, const void* in, const void* xb,
                                          int parity, int64_t j, const EpiCoef<typename PrecTraits<P>::real>& c,
-                                         Spinor<typename PrecTraits<P>::real>& res,
-                                         const Link<typename PrecTraits<P>::real>* sl = nullptr,
-                                         unsigned char* ring = nullptr) {
+                                         Spinor<typename PrecTraits<P>::real>& res, unsigned char* ring = nullptr) {
   Spinor<typename PrecTraits<P>::real> acc;
-  hop_acc<P, R, DAG, GP, SP, AS, BLOCK>(g, gauge, in, parity, j, acc, sl, ring);
+  hop_acc<P, R, DAG, GP, SP, AS, BLOCK>(g, gauge, in, parity, j, acc, ring);
   hop_epilogue<P, DAG, EPI>(g, xb, j, c, acc, res);
 }
 
@@ -525,42 +507,117 @@ template <typename T> __device__ __forceinline__ T norm2_site(const Spinor<T>& r
   return s;
 }
 
-// ---- link staging for the L_s-replicated / multi-RHS hop (n5 >= 4): the n5
-// threads of a 4D site share its eight links (the paper's gauge field reused
-// L_s times, Sec. 3), so a block loads (and for 12-real links rebuilds and, for
-// FP16, converts) each link of its 4D sites once into shared memory and every
-// thread reads them from there instead of repeating that work n5 times.
+// ---- site staging for the L_s-replicated / multi-RHS hop (n5 >= STAGE_MIN_N5): the n5
+// threads of a 4D site share its eight links and neighbours (the paper's gauge
+// field reused L_s times, Sec. 3), so a block loads (and for 12-real links
+// rebuilds and, for FP16, converts) each link of its 4D sites once into shared
+// memory, together with the neighbour's index and the boundary phase, and every
+// thread reads them from there: five 16-byte broadcasts per direction instead of
+// three to nine loads, 36 conversion and rebuild operations and the index
+// arithmetic.
 constexpr int STAGE_MIN_N5 = 4;
-template <int BLOCK> constexpr int stage_sites() { return BLOCK / STAGE_MIN_N5 + 2; }
+// One direction: 18 link reals (row-major), the neighbour's checkerboard index, the phase
+struct StagedDir {
+  float4 q[5];
+};
+constexpr int STAGE_SITE_F4 = 8 * 5 + 1;  // float4 per site: an odd number, so that sites spread over the banks
+__host__ __device__ constexpr int stage_sites(int block, int n5) { return block / n5 + 2; }
 
-// Checkerboard index of the neighbour of x one hop back along a runtime mu.
-__device__ __forceinline__ int64_t back_neighbour_cb(const Geom& g, const Coord& x, int mu) {
-  const int L = mu == 0 ? g.X : mu == 1 ? g.Y : mu == 2 ? g.Z : g.T;
-  const int xm = mu == 0 ? x.c[0] : mu == 1 ? x.c[1] : mu == 2 ? x.c[2] : x.c[3];
-  const uint32_t st = mu == 0 ? 1u : mu == 1 ? (uint32_t)g.st[1] : mu == 2 ? (uint32_t)g.st[2] : (uint32_t)g.st[3];
-  const uint32_t lex = xm == 0 ? x.lex + (uint32_t)(L - 1) * st : x.lex - st;
-  return (int64_t)(lex >> 1);
-}
-
-// Stages the links of the block's 4D sites cb0 .. cb0 + nls - 1 (checkerboard
-// `parity`) into sl[ls * 8 + d]; every thread of the block must call it.
+// Stages the block's 4D sites cb0 .. cb0 + nls - 1 (checkerboard `parity`); every
+// thread of the block must call it.
 template <int P, int R, int BLOCK>
-__device__ __forceinline__ void stage_links(const Geom& g, const void* gauge, int parity, int64_t cb0, int nls,
-                                            Link<typename PrecTraits<P>::real>* sl) {
+__device__ __forceinline__ void stage_block(const Geom& g, const void* gauge, int parity, uint32_t cb0, int nls,
+                                            float4* sm) {
   for (int t = threadIdx.x; t < nls * 8; t += BLOCK) {
     const int ls = t >> 3, d = t & 7, mu = d >> 1;
-    const int64_t cb = cb0 + ls;
-    if (cb >= g.Vh) continue;
-    Link<typename PrecTraits<P>::real> u;
-    if ((d & 1) == 0) {
-      LinkIO<P, R>::load(gauge, g.gstride, parity * 4 + mu, cb, u);
-    } else {
-      const Coord x = cb_to_coord(g, cb, parity);
-      LinkIO<P, R>::load(gauge, g.gstride, (1 - parity) * 4 + mu, back_neighbour_cb(g, x, mu), u);
-    }
-    sl[t] = u;
+    const uint32_t cb = cb0 + ls;
+    if (cb >= (uint32_t)g.Vh) continue;
+    const bool fwd = (d & 1) == 0;
+    const Coord x = cb_to_coord(g, cb, parity);
+    const int L = mu == 0 ? g.X : mu == 1 ? g.Y : mu == 2 ? g.Z : g.T;
+    const int xm = mu == 0 ? x.c[0] : mu == 1 ? x.c[1] : mu == 2 ? x.c[2] : x.c[3];
+    const uint32_t st = mu == 0 ? 1u : mu == 1 ? (uint32_t)g.st[1] : mu == 2 ? (uint32_t)g.st[2] : (uint32_t)g.st[3];
+    const float bc = mu == 0 ? g.bcf[0] : mu == 1 ? g.bcf[1] : mu == 2 ? g.bcf[2] : g.bcf[3];
+    const bool wrap = fwd ? xm == L - 1 : xm == 0;
+    const uint32_t lex = fwd ? (wrap ? x.lex - (uint32_t)(L - 1) * st : x.lex + st)
+                             : (wrap ? x.lex + (uint32_t)(L - 1) * st : x.lex - st);
+    const uint32_t nb = lex >> 1;
+    Link<float> u;
+    LinkIO<P, R>::load(gauge, g.gstride, (fwd ? parity : 1 - parity) * 4 + mu, fwd ? cb : nb, u);
+    float4* q = sm + ls * STAGE_SITE_F4 + d * 5;
+#pragma unroll
+    for (int k = 0; k < 4; k++) q[k] = make_float4(u.v[2 * k].r, u.v[2 * k].i, u.v[2 * k + 1].r, u.v[2 * k + 1].i);
+    q[4] = make_float4(u.v[8].r, u.v[8].i, __uint_as_float(nb), wrap ? bc : 1.f);
   }
   __syncthreads();
+}
+
+// The two hops along MU from the staged site sm, scalar or (SP) spin-paired.
+template <int MU, int P, bool DAG, bool SP, typename Acc>
+__device__ __forceinline__ void hop_dir_staged(Acc& acc, const Geom& g, const float4* sm, uint32_t i5, const void* in) {
+  constexpr int SF = DAG ? +1 : -1;  // forward hop carries (1 + SF gamma_mu)
+#pragma unroll
+  for (int dir = 0; dir < 2; dir++) {
+    const float4* q = sm + (2 * MU + dir) * 5;
+    const float4 last = q[4];
+    const int64_t idx = (int64_t)__float_as_uint(last.z) * g.n5 + i5;
+    Half<float> h;
+    float f = dir == 0 ? load_project<P, MU, SF>(in, g, idx, false, h) : load_project<P, MU, -SF>(in, g, idx, false, h);
+    f *= last.w;
+    Link<float> u;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      const float4 w = q[k];
+      u.v[2 * k] = mk(w.x, w.y);
+      u.v[2 * k + 1] = mk(w.z, w.w);
+    }
+    u.v[8] = mk(last.x, last.y);
+    if constexpr (SP) {
+      SPHalf hp, w;
+#pragma unroll
+      for (int c = 0; c < 3; c++) {
+        hp.r[c] = make_float2(h.v[c].r, h.v[3 + c].r);
+        hp.i[c] = make_float2(h.v[c].i, h.v[3 + c].i);
+      }
+      if (dir == 0) {
+        link_mul_sp<false>(u, hp, w);
+        accumulate_sp<MU, SF>(acc, w, f);
+      } else {
+        link_mul_sp<true>(u, hp, w);
+        accumulate_sp<MU, -SF>(acc, w, f);
+      }
+    } else {
+      Half<float> w;
+      if (dir == 0) {
+        link_mul(u, h, w);
+        accumulate_scaled<MU, SF>(acc, w, f);
+      } else {
+        link_mul_dag(u, h, w);
+        accumulate_scaled<MU, -SF>(acc, w, f);
+      }
+    }
+  }
+}
+
+// H in at slice i5 of the staged site sm.
+template <int P, bool DAG, bool SP>
+__device__ __forceinline__ void hop_acc_staged(const Geom& g, const float4* sm, uint32_t i5, const void* in,
+                                               Spinor<float>& out) {
+  if constexpr (SP) {
+    SPAcc a;
+    sp_zero(a);
+    hop_dir_staged<0, P, DAG, true>(a, g, sm, i5, in);
+    hop_dir_staged<1, P, DAG, true>(a, g, sm, i5, in);
+    hop_dir_staged<2, P, DAG, true>(a, g, sm, i5, in);
+    hop_dir_staged<3, P, DAG, true>(a, g, sm, i5, in);
+    sp_unpack(a, out);
+  } else {
+    zero(out);
+    hop_dir_staged<0, P, DAG, false>(out, g, sm, i5, in);
+    hop_dir_staged<1, P, DAG, false>(out, g, sm, i5, in);
+    hop_dir_staged<2, P, DAG, false>(out, g, sm, i5, in);
+    hop_dir_staged<3, P, DAG, false>(out, g, sm, i5, in);
+  }
 }
 
 // Shared memory of a hop whose neighbour data are copied asynchronously (AS)
@@ -569,17 +626,12 @@ template <int P, int R> constexpr int ring_bytes(int block) {
   else return stage_nslot<P>() * stage_slot_bytes<P, R>() * block;
 }
 
-// One launch computes BLOCK * SPT output sites per block. SPT = 1: one site
-// per thread, any precision. SPT = 2 (FP32 and FP16 storage, not G-parity):
-// thread t of block blk computes sites j0 = blk BLOCK 2 + t and j1 = j0 +
-// BLOCK together in packed FP32x2 arithmetic (hop_pair.cuh), so that every
-// load instruction of a warp stays one coalesced access and the two sites
-// share each FP32 instruction of the hop.
-template <int P, int R, bool DAG, int EPI, int RED, int BLOCK, bool GP, int SPT, bool LS = false, bool SP = false,
+// One thread per output site. LS: links and neighbours staged per 4D site; SP:
+// spin-paired packed arithmetic; AS: neighbour data copied asynchronously.
+template <int P, int R, bool DAG, int EPI, int RED, int BLOCK, bool GP, bool LS = false, bool SP = false,
           bool AS = false>
 __device__ __forceinline__ void hop_body(const HopArgs& A) {
   using T = typename PrecTraits<P>::real;
-  static_assert(SPT == 1 || (SPT == 2 && P != LQCD_F64 && !GP), "two sites per thread: FP32 / FP16, no G-parity");
   overlap_launch();
   if (gate_closed(A.gate)) return;
   int parity = A.out_parity;
@@ -592,129 +644,85 @@ __device__ __forceinline__ void hop_body(const HopArgs& A) {
   char* out = static_cast<char*>(A.out) + (A.full ? parity * A.half_bytes : 0);
   const char* xb = A.x ? static_cast<const char*>(A.x) + (A.full ? parity * A.half_bytes : 0) : nullptr;
   const EpiCoef<T> c = epi_coef<T>(A);
-  const int64_t first = (int64_t)blk * (BLOCK * SPT);
-  if constexpr (SPT == 1) {
-    const int64_t j = first + threadIdx.x;
-    // LS: links staged in shared memory once per 4D site when n5 >= STAGE_MIN_N5
-    const Link<T>* sl = nullptr;
+  const int64_t first = (int64_t)blk * BLOCK;
+  const int64_t j = first + threadIdx.x;
+  // LS: links and neighbours staged in shared memory once per 4D site
+  const float4* site = nullptr;
+  uint32_t i5 = 0;
+  if constexpr (LS) {
+    extern __shared__ float4 staged[];
+    const uint32_t n5 = A.g.n5, cb0 = fdiv((uint32_t)first, A.g.fn5);
+    const int64_t end = first + BLOCK < A.g.nsites ? first + BLOCK : A.g.nsites;
+    stage_block<P, R, BLOCK>(A.g, A.gauge, parity, cb0, (int)(fdiv((uint32_t)end - 1, A.g.fn5) - cb0 + 1), staged);
+    const uint32_t cb = fdiv((uint32_t)j, A.g.fn5);
+    i5 = (uint32_t)j - cb * n5;
+    site = staged + (cb - cb0) * STAGE_SITE_F4;
+  }
+  // AS: the ring of asynchronously copied neighbour data
+  unsigned char* ring = nullptr;
+  if constexpr (AS) {
+    __shared__ __align__(16) unsigned char stage_ring[ring_bytes<P, R>(BLOCK)];
+    ring = stage_ring;
+  }
+  auto hop = [&](Spinor<T>& res) {
     if constexpr (LS) {
-      __shared__ Link<T> staged[stage_sites<BLOCK>() * 8];
-      const int64_t n5 = A.g.n5;
-      if (n5 >= STAGE_MIN_N5) {
-        const int64_t cb0 = first / n5;
-        const int64_t last = (first + BLOCK - 1 < A.g.nsites ? first + BLOCK - 1 : A.g.nsites - 1) / n5;
-        stage_links<P, R, BLOCK>(A.g, A.gauge, parity, cb0, (int)(last - cb0 + 1), staged);
-        if (j < A.g.nsites) sl = staged + (j / n5 - cb0) * 8;
-      }
-    }
-    // AS: the ring of asynchronously copied neighbour data
-    unsigned char* ring = nullptr;
-    if constexpr (AS) {
-      __shared__ __align__(16) unsigned char stage_ring[ring_bytes<P, R>(BLOCK)];
-      ring = stage_ring;
-    }
-    if constexpr (EPI == EPI_M5INV) {
-      // every lane takes part in the fifth-dimension scan; lanes past the end
-      // (whole 4D sites, since L_s divides the block) carry zeros and store nothing
-      static_assert(RED == RED_NONE, "M5op^-1 epilogue without reduction");
-      const bool live = j < A.g.nsites;
-      Spinor<T> res;
-      if (live) hop_site<P, R, DAG, EPI, GP, SP, AS, BLOCK>(A.g, A.gauge, in, xb, parity, j, c, res, sl, ring);
-      else zero(res);
-      const int Ls = A.g.n5;
-      const M5Coef<T> mc = m5_coef<T>(A);
-      m5inv_lanes(res, (int)(threadIdx.x & (unsigned)(Ls - 1)), Ls, A.m5_dagger != 0, mc.a, mc.mf, mc.den_inv);
-      if (live) SpinorIO<P>::store(out, A.g.sstride, j, res);
-      return;
-    }
-    T red = T(0);
-    if (j < A.g.nsites) {
-      Spinor<T> res;
-      hop_site<P, R, DAG, EPI, GP, SP, AS, BLOCK>(A.g, A.gauge, in, xb, parity, j, c, res, sl, ring);
-      if constexpr (RED == RED_CG_UPDATE) {
-        const int64_t ps = A.full ? parity * A.half_bytes : 0, vs = A.full ? parity * A.upd_half_bytes : 0;
-        const int64_t rs = A.full ? parity * A.upd_rs_half_bytes : 0;
-        red = update_site_ap<vec_prec(P), P, rs_prec(P)>(A.g, j, A.red.sys[sys_of(j, A.red.nsys)].alpha,
-                                                         static_cast<const char*>(A.upd_p) + ps, res,
-                                                         static_cast<char*>(A.upd_xs) + vs,
-                                                         static_cast<char*>(A.upd_rs) + rs);
-      } else {
-        SpinorIO<P>::store(out, A.g.sstride, j, res);
-        if constexpr (RED == RED_NORM) red = norm2_site(res);
-      }
-    }
-    if constexpr (RED != RED_NONE) block_reduce_finalize<BLOCK>(red, first, A.red);
-  } else {
-    int64_t j[SPT];
-    bool live[SPT];
-#pragma unroll
-    for (int s = 0; s < SPT; s++) {
-      j[s] = first + s * BLOCK + threadIdx.x;
-      live[s] = j[s] < A.g.nsites;
-    }
-    Spinor<T> acc[SPT];
-    if (live[0]) {
-      // a second site past the end repeats the first one's loads and is not stored
-      PSpinor pa;
-      hop_acc_pair<P, R, DAG>(A.g, A.gauge, in, parity, j[0], live[1] ? j[1] : j[0], pa);
-#pragma unroll
-      for (int k = 0; k < 12; k++) {
-        acc[0].v[k] = pick(pa.v[k], 0);
-        acc[1].v[k] = pick(pa.v[k], 1);
-      }
-    }
-    if constexpr (EPI == EPI_M5INV) {
-      static_assert(RED == RED_NONE, "M5op^-1 epilogue without reduction");
-      const int Ls = A.g.n5;
-#pragma unroll
-      for (int s = 0; s < SPT; s++) {
-        Spinor<T> res;
-        if (live[s]) hop_epilogue<P, DAG, EPI>(A.g, xb, j[s], c, acc[s], res);
-        else zero(res);
-        const M5Coef<T> mc = m5_coef<T>(A);
-        m5inv_lanes(res, (int)(threadIdx.x & (unsigned)(Ls - 1)), Ls, A.m5_dagger != 0, mc.a, mc.mf, mc.den_inv);
-        if (live[s]) SpinorIO<P>::store(out, A.g.sstride, j[s], res);
-      }
+      Spinor<T> acc;
+      hop_acc_staged<P, DAG, SP>(A.g, site, i5, in, acc);
+      hop_epilogue<P, DAG, EPI>(A.g, xb, j, c, acc, res);
     } else {
-      T red[SPT];
-#pragma unroll
-      for (int s = 0; s < SPT; s++) {
-        red[s] = T(0);
-        if (!live[s]) continue;
-        Spinor<T> res;
-        hop_epilogue<P, DAG, EPI>(A.g, xb, j[s], c, acc[s], res);
-        if constexpr (RED == RED_CG_UPDATE) {
-          const int64_t ps = A.full ? parity * A.half_bytes : 0, vs = A.full ? parity * A.upd_half_bytes : 0;
-          const int64_t rs = A.full ? parity * A.upd_rs_half_bytes : 0;
-          red[s] = update_site_ap<vec_prec(P), P, rs_prec(P)>(A.g, j[s], A.red.sys[sys_of(j[s], A.red.nsys)].alpha,
-                                                              static_cast<const char*>(A.upd_p) + ps, res,
-                                                              static_cast<char*>(A.upd_xs) + vs,
-                                                              static_cast<char*>(A.upd_rs) + rs);
-        } else {
-          SpinorIO<P>::store(out, A.g.sstride, j[s], res);
-          if constexpr (RED == RED_NORM) red[s] = norm2_site(res);
-        }
-      }
-      if constexpr (RED != RED_NONE) block_reduce_finalize_n<BLOCK, SPT>(red, first, A.red);
+      hop_site<P, R, DAG, EPI, GP, SP, AS, BLOCK>(A.g, A.gauge, in, xb, parity, j, c, res, ring);
+    }
+  };
+  if constexpr (EPI == EPI_M5INV) {
+    // every lane takes part in the fifth-dimension scan; lanes past the end
+    // (whole 4D sites, since L_s divides the block) carry zeros and store nothing
+    static_assert(RED == RED_NONE, "M5op^-1 epilogue without reduction");
+    const bool live = j < A.g.nsites;
+    Spinor<T> res;
+    if (live) hop(res);
+    else zero(res);
+    const int Ls = A.g.n5;
+    const M5Coef<T> mc = m5_coef<T>(A);
+    m5inv_lanes(res, (int)(threadIdx.x & (unsigned)(Ls - 1)), Ls, A.m5_dagger != 0, mc.a, mc.mf, mc.den_inv);
+    if (live) SpinorIO<P>::store(out, A.g.sstride, j, res);
+    return;
+  }
+  T red = T(0);
+  if (j < A.g.nsites) {
+    Spinor<T> res;
+    hop(res);
+    if constexpr (RED == RED_CG_UPDATE) {
+      const int64_t ps = A.full ? parity * A.half_bytes : 0, vs = A.full ? parity * A.upd_half_bytes : 0;
+      const int64_t rs = A.full ? parity * A.upd_rs_half_bytes : 0;
+      red = update_site_ap<vec_prec(P), P, rs_prec(P)>(A.g, j, A.red.sys[sys_of(j, A.red.nsys)].alpha,
+                                                       static_cast<const char*>(A.upd_p) + ps, res,
+                                                       static_cast<char*>(A.upd_xs) + vs,
+                                                       static_cast<char*>(A.upd_rs) + rs);
+    } else {
+      SpinorIO<P>::store(out, A.g.sstride, j, res);
+      if constexpr (RED == RED_NORM) red = norm2_site(res);
     }
   }
+  if constexpr (RED != RED_NONE) block_reduce_finalize<BLOCK>(red, first, A.red);
 }
 
 // MINB: minimum resident blocks per SM the register allocation must allow
 // (__launch_bounds__; 0 leaves the choice to the compiler), one of the knobs
 // of the launch shapes the tuner times.
 //
-// SPT = -1: one site per thread with the links staged in shared memory (LS);
-// SPT = -2: one site per thread in spin-paired packed arithmetic (SP);
-// SPT = -3 / -4: as 1 / -2 with the neighbour data copied asynchronously
+// KIND 1: the plain hop; -1 / -5: one site per thread with the links and neighbours of each 4D site
+// staged in shared memory (LS), in scalar / spin-paired arithmetic;
+// -2: one site per thread in spin-paired packed arithmetic (SP);
+// -3 / -4: as 1 / -2 with the neighbour data copied asynchronously
 // through a shared-memory ring (AS, hop_async.cuh).
-template <int P, int R, bool DAG, int EPI, int RED, int BLOCK, bool GP = false, int SPT = 1, int MINB = 0>
+template <int P, int R, bool DAG, int EPI, int RED, int BLOCK, bool GP = false, int KIND = 1, int MINB = 0>
 __global__ void __launch_bounds__(BLOCK, MINB) hop_kernel(const HopArgs A) {
-  if constexpr (SPT == -1) hop_body<P, R, DAG, EPI, RED, BLOCK, GP, 1, true>(A);
-  else if constexpr (SPT == -2) hop_body<P, R, DAG, EPI, RED, BLOCK, GP, 1, false, true>(A);
-  else if constexpr (SPT == -3) hop_body<P, R, DAG, EPI, RED, BLOCK, GP, 1, false, false, true>(A);
-  else if constexpr (SPT == -4) hop_body<P, R, DAG, EPI, RED, BLOCK, GP, 1, false, true, true>(A);
-  else hop_body<P, R, DAG, EPI, RED, BLOCK, GP, SPT>(A);
+  if constexpr (KIND == -1) hop_body<P, R, DAG, EPI, RED, BLOCK, GP, true>(A);
+  else if constexpr (KIND == -2) hop_body<P, R, DAG, EPI, RED, BLOCK, GP, false, true>(A);
+  else if constexpr (KIND == -3) hop_body<P, R, DAG, EPI, RED, BLOCK, GP, false, false, true>(A);
+  else if constexpr (KIND == -4) hop_body<P, R, DAG, EPI, RED, BLOCK, GP, false, true, true>(A);
+  else if constexpr (KIND == -5) hop_body<P, R, DAG, EPI, RED, BLOCK, GP, true, true>(A);
+  else hop_body<P, R, DAG, EPI, RED, BLOCK, GP>(A);
 }
 
 }  // namespace lqcd

@@ -6,23 +6,28 @@
 
 namespace lqcd {
 
-template <int P, int R, bool DAG, int EPI, int RED, bool GP, int BLOCK, int SPT, int MINB>
+template <int P, int R, bool DAG, int EPI, int RED, bool GP, int BLOCK, int KIND, int MINB>
 static int launch_hop_shape(HopArgs a, cudaStream_t s) {
-  constexpr int SITES = SPT < 0 ? 1 : SPT;  // SPT -1 .. -4: one site per thread
-  const int64_t nb = (a.g.nsites + BLOCK * SITES - 1) / (BLOCK * SITES);
+  size_t shared = 0;
+  if constexpr (KIND == -1 || KIND == -5) {
+    // the staged hop shares a site among n5 threads; without enough of them it is the plain one
+    if (a.g.n5 < STAGE_MIN_N5) return launch_hop_shape<P, R, DAG, EPI, RED, GP, HOP_BLOCK, 1, 0>(a, s);
+    shared = (size_t)stage_sites(BLOCK, a.g.n5) * STAGE_SITE_F4 * sizeof(float4);
+  }
+  const int64_t nb = (a.g.nsites + BLOCK - 1) / BLOCK;
   a.blocks_per_parity = (int)nb;
   const int64_t grid = a.full ? 2 * nb : nb;
   if (grid == 0) return LQCD_OK;
-  if constexpr (SPT <= -3) {
-    // the staged hop's ring: ask for the largest shared-memory carveout so that
+  if constexpr (KIND == -3 || KIND == -4) {
+    // the ring of asynchronous copies: ask for the largest shared-memory carveout so that
     // MINB blocks of it fit an SM
-    static const cudaError_t carve = cudaFuncSetAttribute(hop_kernel<P, R, DAG, EPI, RED, BLOCK, GP, SPT, MINB>,
+    static const cudaError_t carve = cudaFuncSetAttribute(hop_kernel<P, R, DAG, EPI, RED, BLOCK, GP, KIND, MINB>,
                                                           cudaFuncAttributePreferredSharedMemoryCarveout,
                                                           (int)cudaSharedmemCarveoutMaxShared);
     if (carve != cudaSuccess) return cuda_fail(carve, "hop_kernel: shared-memory carveout");
   }
-  const cudaError_t e = launch_overlapped<HopArgs>(hop_kernel<P, R, DAG, EPI, RED, BLOCK, GP, SPT, MINB>,
-                                                   (unsigned)grid, BLOCK, s, a);
+  const cudaError_t e = launch_overlapped<HopArgs>(hop_kernel<P, R, DAG, EPI, RED, BLOCK, GP, KIND, MINB>,
+                                                   (unsigned)grid, BLOCK, shared, s, a);
   if (e != cudaSuccess) return cuda_fail(e, "hop_kernel");
   return after_launch("hop_kernel");
 }
@@ -30,8 +35,8 @@ static int launch_hop_shape(HopArgs a, cudaStream_t s) {
 template <int P, int R, bool DAG, int EPI, int RED, bool GP>
 static int launch_hop_index(int idx, const HopArgs& a, cudaStream_t s) {
   switch (idx) {
-#define LQCD_HOP_CASE(I, B, S, M) \
-  case I: return launch_hop_shape<P, R, DAG, EPI, RED, GP, B, S, M>(a, s);
+#define LQCD_HOP_CASE(I, B, K, M) \
+  case I: return launch_hop_shape<P, R, DAG, EPI, RED, GP, B, K, M>(a, s);
     LQCD_HOP_SHAPES(LQCD_HOP_CASE)
 #undef LQCD_HOP_CASE
   }

@@ -222,16 +222,9 @@ __device__ __forceinline__ void hop_acc_async(const Geom& g, const void* gauge, 
   }
   if constexpr (SP) {
     SPAcc a;
-#pragma unroll
-    for (int c = 0; c < 3; c++) a.ur[c] = a.ui[c] = a.lr[c] = a.li[c] = make_float2(0.f, 0.f);
+    sp_zero(a);
     stage_step<P, R, BLOCK, NSLOT, DAG, true, 0>(ring, a, g, gauge, in, x, cb, i5, parity);
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-      out.v[c] = mk(a.ur[c].x, a.ui[c].x);
-      out.v[3 + c] = mk(a.ur[c].y, a.ui[c].y);
-      out.v[6 + c] = mk(a.lr[c].x, a.li[c].x);
-      out.v[9 + c] = mk(a.lr[c].y, a.li[c].y);
-    }
+    sp_unpack(a, out);
   } else {
     zero(out);
     stage_step<P, R, BLOCK, NSLOT, DAG, false, 0>(ring, out, g, gauge, in, x, cb, i5, parity);

@@ -36,7 +36,8 @@ inline int64_t round_up(int64_t a, int64_t b) { return (a + b - 1) / b * b; }
 // solver's conditional graph it loses 7 % (158 -> 169 us an iteration), so a captured
 // launch is an ordinary one.
 template <typename Arg>
-inline cudaError_t launch_overlapped(void (*kernel)(Arg), unsigned grid, unsigned block, cudaStream_t s, const Arg& arg) {
+inline cudaError_t launch_overlapped(void (*kernel)(Arg), unsigned grid, unsigned block, size_t shared,
+                                     cudaStream_t s, const Arg& arg) {
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   const cudaError_t e = cudaStreamIsCapturing(s, &capture);
   if (e != cudaSuccess) return e;
@@ -46,6 +47,7 @@ inline cudaError_t launch_overlapped(void (*kernel)(Arg), unsigned grid, unsigne
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = shared;
   cfg.stream = s;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
@@ -725,38 +727,6 @@ __device__ __forceinline__ void block_reduce_finalize(V v, int64_t block_first_g
     }
   }
   last_block_finalize<BLOCK>(rc, sh);
-}
-
-// block_reduce_finalize for SPT values per thread: value s of thread t belongs to
-// global index block_first_gid + s BLOCK + t (the layout of the two-site hop).
-template <int BLOCK, int SPT, typename V>
-__device__ __forceinline__ void block_reduce_finalize_n(const V (&v)[SPT], int64_t block_first_gid,
-                                                        const ReduceCtx& rc) {
-  if constexpr (SPT == 1) {
-    block_reduce_finalize<BLOCK>(v[0], block_first_gid, rc);
-  } else {
-    const int nsys = rc.nsys;
-    if (nsys == 1) {
-      V sum = v[0];
-#pragma unroll
-      for (int s = 1; s < SPT; s++) sum += v[s];
-      block_reduce_finalize<BLOCK>(sum, block_first_gid, rc);
-      return;
-    }
-    __shared__ double sh[BLOCK];
-    __shared__ V shv[BLOCK * SPT];
-    const int tid = threadIdx.x;
-#pragma unroll
-    for (int s = 0; s < SPT; s++) shv[s * BLOCK + tid] = v[s];
-    __syncthreads();
-    if (tid < nsys) {
-      const int first = (int)((tid - block_first_gid % nsys + nsys) % nsys);
-      double acc = 0.0;
-      for (int k = first; k < BLOCK * SPT; k += nsys) acc += (double)shv[k];
-      rc.partials[(int64_t)tid * gridDim.x + blockIdx.x] = acc;
-    }
-    last_block_finalize<BLOCK>(rc, sh);
-  }
 }
 
 // System index of a site index j = cb * n5 + i5.

@@ -153,10 +153,11 @@ int tune_hop_shapes(const HopKey& k, const std::function<int(int)>& launch, cuda
   int st = LQCD_OK;
   for (int i = 0; i < HOP_SHAPES && st == LQCD_OK; i++) {
     t[i] = 3.0e38f;
-    st = launch(i);
+    if (hop_shape_applies(i, k.n5)) st = launch(i);
   }
   for (int r = 0; r < ROUNDS && st == LQCD_OK; r++) {
     for (int i = 0; i < HOP_SHAPES && st == LQCD_OK; i++) {
+      if (!hop_shape_applies(i, k.n5)) continue;
       cudaEventRecord(e0, s);
       for (int q = 0; q < PAIR && st == LQCD_OK; q++) st = launch(i);
       cudaEventRecord(e1, s);
