@@ -44,10 +44,24 @@ def _ptr(x) -> Optional[int]:
     return x.data_ptr()  # torch tensor
 
 
+_torch = None  # torch, and its raw-stream query, once a call has needed them
+
+
+def _current_stream() -> Optional[int]:
+    global _torch
+    if _torch is None:
+        import torch
+        _torch = torch, getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    torch, raw = _torch
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream or None
+    # the handle without a Stream object around it: 0.5 instead of 2.9 us per call
+    return raw(torch.cuda.current_device()) or None
+
+
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream or None
+        return _current_stream()
     if isinstance(stream, int):
         return stream or None
     return stream.cuda_stream or None
