@@ -46,16 +46,18 @@ __device__ __forceinline__ double init_site(const Geom& g, int64_t j, const doub
   return site_norm2(b);
 }
 
-// x_s += alpha p; r_s -= alpha Ap with Ap given in registers; returns |r_s|^2 (in VF's type)
+// x = x_s + alpha p, r = r_s - alpha Ap with Ap given in registers; returns |r|^2 (in VF's type)
 template <int VF, int SF, int RF = VF, typename TA>
-__device__ __forceinline__ typename PrecTraits<VF>::real update_site_ap(const Geom& g, int64_t j, double alpha_d, const void* p_,
-                                                 const Spinor<TA>& ap, void* xs, void* rs) {
+__device__ __forceinline__ typename PrecTraits<VF>::real updated_site(const Geom& g, int64_t j, double alpha_d,
+                                                                      const void* p_, const Spinor<TA>& ap,
+                                                                      const void* xs, const void* rs,
+                                                                      Spinor<typename PrecTraits<VF>::real>& x,
+                                                                      Spinor<typename PrecTraits<VF>::real>& r) {
   using TV = typename PrecTraits<VF>::real;
   using TS = typename PrecTraits<SF>::real;
   const TV alpha = (TV)alpha_d;
   Spinor<TS> p;
   SpinorIO<SF>::load(p_, g.sstride, j, p);
-  Spinor<TV> x, r;
   SpinorIO<VF>::load(xs, g.sstride, j, x);
   SpinorIO<RF>::load(rs, g.sstride, j, r);
 #pragma unroll
@@ -63,9 +65,19 @@ __device__ __forceinline__ typename PrecTraits<VF>::real update_site_ap(const Ge
     x.v[k] = mk(fma(alpha, (TV)p.v[k].r, x.v[k].r), fma(alpha, (TV)p.v[k].i, x.v[k].i));
     r.v[k] = mk(fma(-alpha, (TV)ap.v[k].r, r.v[k].r), fma(-alpha, (TV)ap.v[k].i, r.v[k].i));
   }
+  return site_norm2(r);
+}
+
+// x_s += alpha p; r_s -= alpha Ap with Ap given in registers; returns |r_s|^2 (in VF's type)
+template <int VF, int SF, int RF = VF, typename TA>
+__device__ __forceinline__ typename PrecTraits<VF>::real update_site_ap(const Geom& g, int64_t j, double alpha_d,
+                                                                        const void* p_, const Spinor<TA>& ap, void* xs,
+                                                                        void* rs) {
+  Spinor<typename PrecTraits<VF>::real> x, r;
+  const auto red = updated_site<VF, SF, RF>(g, j, alpha_d, p_, ap, xs, rs, x, r);
   SpinorIO<VF>::store(xs, g.sstride, j, x);
   SpinorIO<RF>::store(rs, g.sstride, j, r);
-  return site_norm2(r);
+  return red;
 }
 
 // x_s += alpha p; r_s -= alpha Ap; returns |r_s|^2 (in VF's type)

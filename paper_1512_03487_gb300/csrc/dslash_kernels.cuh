@@ -687,23 +687,39 @@ __device__ __forceinline__ void hop_body(const HopArgs& A) {
     if (live) SpinorIO<P>::store(out, A.g.sstride, j, res);
     return;
   }
-  T red = T(0);
-  if (j < A.g.nsites) {
-    Spinor<T> res;
-    hop(res);
-    if constexpr (RED == RED_CG_UPDATE) {
-      const int64_t ps = A.full ? parity * A.half_bytes : 0, vs = A.full ? parity * A.upd_half_bytes : 0;
-      const int64_t rs = A.full ? parity * A.upd_rs_half_bytes : 0;
-      red = update_site_ap<vec_prec(P), P, rs_prec(P)>(A.g, j, A.red.sys[sys_of(j, A.red.nsys)].alpha,
-                                                       static_cast<const char*>(A.upd_p) + ps, res,
-                                                       static_cast<char*>(A.upd_xs) + vs,
-                                                       static_cast<char*>(A.upd_rs) + rs);
-    } else {
-      SpinorIO<P>::store(out, A.g.sstride, j, res);
-      if constexpr (RED == RED_NORM) red = norm2_site(res);
+  const bool live = j < A.g.nsites;
+  Spinor<T> res;
+  if constexpr (RED == RED_CG_UPDATE) {
+    const int64_t ps = A.full ? parity * A.half_bytes : 0, vs = A.full ? parity * A.upd_half_bytes : 0;
+    const int64_t rs = A.full ? parity * A.upd_rs_half_bytes : 0;
+    char* xs_p = static_cast<char*>(A.upd_xs) + vs;
+    char* rs_p = static_cast<char*>(A.upd_rs) + rs;
+    Spinor<typename PrecTraits<vec_prec(P)>::real> x, r;
+    T red = T(0);
+    if (live) {
+      hop(res);
+      red = updated_site<vec_prec(P), P, rs_prec(P)>(A.g, j, A.red.sys[sys_of(j, A.red.nsys)].alpha,
+                                                     static_cast<const char*>(A.upd_p) + ps, res, xs_p, rs_p, x, r);
     }
+    block_reduce_finalize<BLOCK>(red, first, A.red, [&]() {
+      if (!live) return;
+      SpinorIO<vec_prec(P)>::store(xs_p, A.g.sstride, j, x);
+      SpinorIO<rs_prec(P)>::store(rs_p, A.g.sstride, j, r);
+    });
+  } else if constexpr (RED == RED_NORM) {
+    T red = T(0);
+    if (live) {
+      hop(res);
+      red = norm2_site(res);
+    }
+    block_reduce_finalize<BLOCK>(red, first, A.red, [&]() {
+      if (live) SpinorIO<P>::store(out, A.g.sstride, j, res);
+    });
+  } else {
+    if (!live) return;
+    hop(res);
+    SpinorIO<P>::store(out, A.g.sstride, j, res);
   }
-  if constexpr (RED != RED_NONE) block_reduce_finalize<BLOCK>(red, first, A.red);
 }
 
 // MINB: minimum resident blocks per SM the register allocation must allow
