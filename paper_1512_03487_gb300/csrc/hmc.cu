@@ -343,31 +343,47 @@ __device__ __forceinline__ void exp_coefficients(cpx<double> t, cpx<double> s, c
   }
 }
 
-// U <- exp(i eps P) U per link. exp(A), A = i eps P, is its Taylor polynomial
-// reduced to second degree in A by the characteristic equation (any 3x3 matrix
-// P): one product for A^2, scalars, and one product with U, about 480 FMA
-// instead of the 2,150 of a degree-16 Horner scheme on matrices, which the FP64
-// pipe bounds either way. Degree 13 up to |A|_F = 1/4 (molecular-dynamics steps
-// stay there), 20 up to 1, truncation below 1e-19; a larger A is halved until
-// |A|_F <= 1 and the exponential squared back.
-__global__ void __launch_bounds__(HMC_BLOCK) exp_update_kernel(void* U, const void* P, Geom g, double eps) {
-  const int64_t t = (int64_t)blockIdx.x * HMC_BLOCK + threadIdx.x;
-  if (t >= 8 * (int64_t)g.Vh) return;
-  const int blk = (int)(t / g.Vh);  // parity * 4 + mu
-  const int64_t cb = t - (int64_t)blk * g.Vh;
-  M3 A, A2, u, E;
-  LinkIO<LQCD_F64, 18>::load(P, g.gstride, blk, cb, A);
-  double n2 = 0.0;
+// The same for exp(i H), H^3 = t H^2 - s H + d with t, s, d real (H Hermitian): 6 FMA a step.
+template <int N>
+__device__ __forceinline__ void exp_coefficients(double t, double s, double d, cpx<double> q[3]) {
+  cpx<double> c[N + 1];  // i^n / n!, folded at compile time
+  c[0] = mk(1.0, 0.0);
 #pragma unroll
-  for (int k = 0; k < 9; k++) {
-    A.v[k] = mk(-eps * A.v[k].i, eps * A.v[k].r);  // i eps P
-    n2 = fma(A.v[k].r, A.v[k].r, fma(A.v[k].i, A.v[k].i, n2));
+  for (int n = 1; n <= N; n++) c[n] = mk(-c[n - 1].i / n, c[n - 1].r / n);
+  q[2] = c[N];
+  q[1] = c[N - 1];
+  q[0] = c[N - 2];
+#pragma unroll
+  for (int n = N - 3; n >= 0; n--) {
+    const cpx<double> top = q[2];
+    q[2] = mk(fma(t, top.r, q[1].r), fma(t, top.i, q[1].i));
+    q[1] = mk(fma(-s, top.r, q[0].r), fma(-s, top.i, q[0].i));
+    q[0] = mk(fma(d, top.r, c[n].r), fma(d, top.i, c[n].i));
   }
+}
+
+// Halvings that bring |A|_F^2 = n2 to 1 or below; n2 becomes that of the halved A.
+__device__ __forceinline__ int halvings(double& n2) {
   int s = 0;
   while (n2 > 1.0 && s < 60) {
     n2 *= 0.25;
     s++;
   }
+  return s;
+}
+
+__device__ __forceinline__ double abs2(cpx<double> a) { return fma(a.r, a.r, a.i * a.i); }
+
+// E = exp(2^-s A), A = i eps P, for any matrix P; returns s.
+__device__ __forceinline__ int exp_general(const M3& P, double eps, M3& E) {
+  M3 A, A2;
+  double n2 = 0.0;
+#pragma unroll
+  for (int k = 0; k < 9; k++) {
+    A.v[k] = mk(-eps * P.v[k].i, eps * P.v[k].r);  // i eps P
+    n2 = fma(A.v[k].r, A.v[k].r, fma(A.v[k].i, A.v[k].i, n2));
+  }
+  const int s = halvings(n2);
   if (s > 0) {
     const double sc = ldexp(1.0, -s);
 #pragma unroll
@@ -390,15 +406,91 @@ __global__ void __launch_bounds__(HMC_BLOCK) exp_update_kernel(void* U, const vo
     const cpx<double> e = cmadd(k % 4 == 0 ? q[0] : mk(0.0, 0.0), q[1], A.v[k]);
     E.v[k] = cmadd(e, q[2], A2.v[k]);
   }
+  return s;
+}
+
+// The same for a Hermitian P, from its diagonal and upper triangle: with H = 2^-s
+// eps P the invariants are real, H^2 is Hermitian, and the elements rc and cr of
+// q1 H + q2 H^2 share their products.
+__device__ __forceinline__ int exp_hermitian(const M3& P, double eps, M3& E) {
+  double d[3] = {eps * P.v[0].r, eps * P.v[4].r, eps * P.v[8].r};
+  cpx<double> x = eps * P.v[1], y = eps * P.v[2], z = eps * P.v[5];  // H_01, H_02, H_12
+  double xx = abs2(x), yy = abs2(y), zz = abs2(z);
+  double n2 = fma(d[0], d[0], fma(d[1], d[1], fma(d[2], d[2], 2.0 * (xx + yy + zz))));
+  const int s = halvings(n2);
+  if (s > 0) {
+    const double sc = ldexp(1.0, -s), sc2 = sc * sc;
+#pragma unroll
+    for (int k = 0; k < 3; k++) d[k] *= sc;
+    x = sc * x;
+    y = sc * y;
+    z = sc * z;
+    xx *= sc2;
+    yy *= sc2;
+    zz *= sc2;
+  }
+  const double K[3] = {fma(d[0], d[0], xx + yy), fma(d[1], d[1], xx + zz), fma(d[2], d[2], yy + zz)};
+  const cpx<double> xz = cmul(x, z);
+  const cpx<double> kx = cmadd_conj((d[0] + d[1]) * x, z, y);  // (H^2)_01 = (d0 + d1) x + conj(z) y
+  const cpx<double> ky = (d[0] + d[2]) * y + xz;
+  const cpx<double> kz = cmadd_conj((d[1] + d[2]) * z, x, y);  // (H^2)_12 = (d1 + d2) z + conj(x) y
+  const double tr = d[0] + d[1] + d[2];
+  const double sec = fma(d[0], d[1], fma(d[2], d[0] + d[1], -(xx + yy + zz)));
+  double det = fma(2.0, fma(xz.r, y.r, xz.i * y.i), d[0] * fma(d[1], d[2], -zz));  // 2 Re(x z conj(y))
+  det = fma(-d[1], yy, fma(-d[2], xx, det));
+  cpx<double> q[3];
+  if (n2 <= 0.0625) exp_coefficients<13>(tr, sec, det, q);
+  else exp_coefficients<20>(tr, sec, det, q);
+#pragma unroll
+  for (int k = 0; k < 3; k++)
+    E.v[4 * k] = mk(fma(q[2].r, K[k], fma(q[1].r, d[k], q[0].r)), fma(q[2].i, K[k], fma(q[1].i, d[k], q[0].i)));
+  auto pair = [&](cpx<double> h, cpx<double> k, cpx<double>& up, cpx<double>& low) {
+    const double a = fma(q[2].r, k.r, q[1].r * h.r), b = fma(q[2].i, k.i, q[1].i * h.i);
+    const double c = fma(q[2].r, k.i, q[1].r * h.i), e = fma(q[2].i, k.r, q[1].i * h.r);
+    up = mk(a - b, c + e);
+    low = mk(a + b, e - c);
+  };
+  pair(x, kx, E.v[1], E.v[3]);
+  pair(y, ky, E.v[2], E.v[6]);
+  pair(z, kz, E.v[5], E.v[7]);
+  return s;
+}
+
+__device__ __forceinline__ bool is_hermitian(const M3& p) {
+  bool h = p.v[0].i == 0.0 && p.v[4].i == 0.0 && p.v[8].i == 0.0;
+#pragma unroll
+  for (int e = 0; e < 3; e++) {
+    const int r = e == 2 ? 1 : 0, c = e == 0 ? 1 : 2;
+    h = h && p.v[3 * r + c].r == p.v[3 * c + r].r && p.v[3 * r + c].i == -p.v[3 * c + r].i;
+  }
+  return h;
+}
+
+// U <- exp(i eps P) U per link. exp(A), A = i eps P, is its Taylor polynomial
+// reduced to second degree in A by the characteristic equation: one product for
+// A^2, scalars, and one product with U, about 480 FMA instead of the 2,150 of a
+// degree-16 Horner scheme on matrices, which the FP64 pipe bounds either way. A P
+// that is Hermitian to the last bit, as the momenta are (the forces write one
+// triangle and mirror it), takes about 290 (16^4: 253 -> 149 us). Degree 13 up to |A|_F = 1/4
+// (molecular-dynamics steps stay there), 20 up to 1, truncation below 1e-19; a
+// larger A is halved until |A|_F <= 1 and the exponential squared back.
+__global__ void __launch_bounds__(HMC_BLOCK) exp_update_kernel(void* U, const void* P, Geom g, double eps) {
+  const int64_t t = (int64_t)blockIdx.x * HMC_BLOCK + threadIdx.x;
+  if (t >= 8 * (int64_t)g.Vh) return;
+  const int blk = (int)(t / g.Vh);  // parity * 4 + mu
+  const int64_t cb = t - (int64_t)blk * g.Vh;
+  M3 p, E, u, w;
+  LinkIO<LQCD_F64, 18>::load(P, g.gstride, blk, cb, p);
+  const int s = is_hermitian(p) ? exp_hermitian(p, eps, E) : exp_general(p, eps, E);
   for (int k = 0; k < s; k++) {
-    m_mul(E, E, A2);
-    E = A2;
+    m_mul(E, E, w);
+    E = w;
   }
   LinkIO<LQCD_F64, 18>::load(U, g.gstride, blk, cb, u);
-  m_mul(E, u, A2);
+  m_mul(E, u, w);
   double2* base = static_cast<double2*>(U) + (int64_t)blk * 9 * g.gstride + cb;
 #pragma unroll
-  for (int k = 0; k < 9; k++) base[k * g.gstride] = make_double2(A2.v[k].r, A2.v[k].i);
+  for (int k = 0; k < 9; k++) base[k * g.gstride] = make_double2(w.v[k].r, w.v[k].i);
 }
 
 // sum over the 4 links of a site of tr(P^2) / 2 = |P|_F^2 / 2 (P Hermitian), reduced

@@ -63,6 +63,37 @@ def test_link_update_around_its_thresholds(L, norm, hermitian):
     assert _rel(F.gauge_to_host(Ud, lat, 0, 18), expect) <= 1e-13
 
 
+# Links side by side with a Hermitian P (one triangle used), one that is so only up to its
+# last bits and any matrix: the same tolerance as above for each. A NaN or an asymmetry that
+# stands in the lower triangle alone counts.
+@pytest.mark.parametrize("norm", [0.2, 0.9, 3.0])
+def test_link_update_of_hermitian_and_general_momenta_side_by_side(L, norm):
+    from scipy.linalg import expm
+    F = L.fields
+    dims = (2, 4, 2, 6)
+    lat = L.lattice(dims)
+    U = gauge_field(dims, "haar", 1821)
+    n = U.size // 9
+    rng = make_rng(1822)
+    P = rng.standard_normal((n, 3, 3)) + 1j * rng.standard_normal((n, 3, 3))
+    P *= (norm / 0.5 / np.linalg.norm(P, axis=(1, 2)))[:, None, None]
+    kind = rng.integers(0, 3, n)
+    herm = 0.5 * (P + P.conj().transpose(0, 2, 1))
+    P = np.where((kind < 2)[:, None, None], herm, P)
+    P[kind == 1, 2, 0] *= 1.0 + 4e-16
+    expect = np.einsum("nij,njk->nik", np.stack([expm(0.5j * p) for p in P]), U.reshape(n, 3, 3))
+    bad = np.flatnonzero(kind == 0)[:2]
+    P[bad[0], 2, 1] = np.nan
+    P[bad[1], 1, 1] += 1e-3j
+    expect[bad[1]] = expm(0.5j * P[bad[1]]) @ U.reshape(n, 3, 3)[bad[1]]
+    Ud = F.gauge_to_device(U, lat, 0, 18)
+    L.lqcd_gauge_exp_update(Ud, F.gauge_to_device(P.reshape(U.shape), lat, 0, 18), 0.5, lat)
+    got = F.gauge_to_host(Ud, lat, 0, 18).reshape(n, 3, 3)
+    assert np.isnan(got[bad[0]]).all()
+    keep = np.arange(n) != bad[0]
+    assert _rel(got[keep], expect[keep]) <= 1e-13
+
+
 # sums of at most a hundred products, as in the oracle: 1e-12 as for the full lattices
 @pytest.mark.parametrize("recon", [18, 12])
 @pytest.mark.parametrize("dims", [(2, 2, 2, 2), (4, 2, 2, 2), (2, 6, 2, 6)])
