@@ -62,6 +62,8 @@ struct VecArgs {
   double* r64;        // FP64 residual
   const double* ax64; // FP64 A x
   const void* ax32;   // FP32 A x_s of the intermediate replacement (FP32 field)
+  const void* b32;    // k_init: FP32 source in place of b64, or null
+  void* r32;          // CGNR with FP32 arithmetic inside: FP32 residual in place of r64, or null
   void* xs;           // sloppy-vector solution increment (VF)
   void* rs;           // sloppy-vector residual (rs_prec)
   void* p;            // search direction (SF)
@@ -88,14 +90,43 @@ __device__ __forceinline__ bool vec_site(const VecArgs& a, int& parity, int64_t&
 // r = b, r_s = b, p = b, x_s = 0, x = 0; |b|^2 -> initial state
 template <int VF, int SF>
 __global__ void __launch_bounds__(BLAS_BLOCK) k_init(VecArgs a) {
+  using TV = typename PrecTraits<VF>::real;
+  using TS = typename PrecTraits<SF>::real;
   int parity;
   int64_t j, first;
   double red = 0.0;
-  if (vec_site(a, parity, j, first))
-    red = init_site<VF, SF, rs_prec(SF)>(a.g, j, PAR_PTR(a.b64, a.hb64), PAR_PTR(a.r64, a.hb64),
-                                         PAR_PTR(a.x64, a.hb64), PAR_PTR(a.rs, a.hbr), PAR_PTR(a.xs, a.hbv),
-                                         PAR_PTR(a.p, a.hbs));
-  block_reduce_finalize<BLAS_BLOCK>(red, first, a.red);
+  Spinor<double> b;
+  const bool live = vec_site(a, parity, j, first);
+  if (live) {
+    if (a.b32) {
+      Spinor<float> f;
+      SpinorIO<LQCD_F32>::load(PAR_PTR(a.b32, a.hbv), a.g.sstride, j, f);
+      convert(f, b);
+    } else {
+      SpinorIO<LQCD_F64>::load(PAR_PTR(a.b64, a.hb64), a.g.sstride, j, b);
+    }
+    red = site_norm2(b);
+  }
+  block_reduce_finalize<BLAS_BLOCK>(red, first, a.red, [&]() {
+    if (!live) return;
+    Spinor<TV> v;
+    convert(b, v);
+    if (a.r32) {
+      Spinor<float> f;
+      convert(b, f);
+      SpinorIO<LQCD_F32>::store(PAR_PTR(a.r32, a.hbv), a.g.sstride, j, f);
+    } else {
+      SpinorIO<LQCD_F64>::store(PAR_PTR(a.r64, a.hb64), a.g.sstride, j, b);
+    }
+    SpinorIO<rs_prec(SF)>::store(PAR_PTR(a.rs, a.hbr), a.g.sstride, j, v);
+    Spinor<TS> s;
+    convert(b, s);
+    SpinorIO<SF>::store(PAR_PTR(a.p, a.hbs), a.g.sstride, j, s);
+    zero(b);
+    zero(v);
+    SpinorIO<LQCD_F64>::store(PAR_PTR(a.x64, a.hb64), a.g.sstride, j, b);
+    SpinorIO<VF>::store(PAR_PTR(a.xs, a.hbv), a.g.sstride, j, v);
+  });
 }
 
 // p = r_s + beta p
@@ -129,51 +160,55 @@ __global__ void __launch_bounds__(BLAS_BLOCK) k_residual(VecArgs a) {
                                 PAR_PTR(a.rs, a.hbr));
   block_reduce_finalize<BLAS_BLOCK>(red, first, a.red);
 }
-// dst = src between formats (the CGNR start: M^dag b in FP32 arithmetic)
-template <int DP, int SP>
-__global__ void __launch_bounds__(BLAS_BLOCK) k_copy_field(VecArgs a, void* dst, const void* src) {
-  int parity;
-  int64_t j, first;
-  if (!vec_site(a, parity, j, first)) return;
-  const int64_t hd = parity * (int64_t)cb_spinor_bytes(a.g, DP), hs = parity * (int64_t)cb_spinor_bytes(a.g, SP);
-  Spinor<typename PrecTraits<SP>::real> v;
-  SpinorIO<SP>::load(static_cast<const char*>(src) + hs, a.g.sstride, j, v);
-  Spinor<typename PrecTraits<DP>::real> w;
-  convert(v, w);
-  SpinorIO<DP>::store(static_cast<char*>(dst) + hd, a.g.sstride, j, w);
-}
 
-// CGNR: out = b - mx in FP64 and |b - mx|^2 per system (a.red, FIN_STORE);
-// with mx null only |b|^2 (out may alias mx)
-__global__ void __launch_bounds__(BLAS_BLOCK) k_b_minus(VecArgs a, double* out, const double* mx) {
+// CGNR: b - mx (b itself with mx null) in FP64, |b - mx|^2 per system (a.red,
+// FIN_STORE), and the vector stored to out in FP64 (which may alias mx) or, rounded
+// once, in FP32; out may be null. The FP32 form is what the FP32 operator reads next:
+// without it the vector went through memory twice more (24^3 x 48: 46 + 18 us).
+template <int OP>
+__global__ void __launch_bounds__(BLAS_BLOCK) k_b_minus(VecArgs a, void* out, const double* mx) {
   int parity;
   int64_t j, first;
   double red = 0.0;
-  if (vec_site(a, parity, j, first)) {
-    const int64_t h = parity * a.hb64;
-    Spinor<double> b, m;
-    SpinorIO<LQCD_F64>::load(reinterpret_cast<const char*>(a.b64) + h, a.g.sstride, j, b);
+  Spinor<double> b;
+  const bool live = vec_site(a, parity, j, first);
+  if (live) {
+    SpinorIO<LQCD_F64>::load(PAR_PTR(a.b64, a.hb64), a.g.sstride, j, b);
     if (mx) {
-      SpinorIO<LQCD_F64>::load(reinterpret_cast<const char*>(mx) + h, a.g.sstride, j, m);
+      Spinor<double> m;
+      SpinorIO<LQCD_F64>::load(PAR_PTR(mx, a.hb64), a.g.sstride, j, m);
 #pragma unroll
       for (int k = 0; k < 12; k++) b.v[k] = b.v[k] - m.v[k];
-      SpinorIO<LQCD_F64>::store(reinterpret_cast<char*>(out) + h, a.g.sstride, j, b);
     }
     red = site_norm2(b);
   }
-  block_reduce_finalize<BLAS_BLOCK>(red, first, a.red);
+  block_reduce_finalize<BLAS_BLOCK>(red, first, a.red, [&]() {
+    if (!live || !out) return;
+    Spinor<typename PrecTraits<OP>::real> o;
+    convert(b, o);
+    SpinorIO<OP>::store(PAR_PTR(out, OP == LQCD_F64 ? a.hb64 : a.hbv), a.g.sstride, j, o);
+  });
 }
 
-// CGNR: r = M^dag (b - M x) from its FP32-arithmetic value (a.ax32) -> FP64 r,
-// r_s; |r|^2 -> FIN_RELIABLE (exit decided by the FP64 |b - M x|^2)
+// CGNR: r = M^dag (b - M x) in its FP32-arithmetic value (a.r32) -> r_s;
+// |r|^2 -> FIN_RELIABLE (exit decided by the FP64 |b - M x|^2)
 template <int VF, int RF>
 __global__ void __launch_bounds__(BLAS_BLOCK) k_residual32(VecArgs a) {
+  using TV = typename PrecTraits<VF>::real;
   int parity;
   int64_t j, first;
-  typename PrecTraits<VF>::real red = 0;
-  if (vec_site(a, parity, j, first))
-    red = residual32_site<VF, RF>(a.g, j, PAR_PTR(a.ax32, a.hbv), PAR_PTR(a.r64, a.hb64), PAR_PTR(a.rs, a.hbr));
-  block_reduce_finalize<BLAS_BLOCK>(red, first, a.red);
+  TV red = 0;
+  Spinor<TV> r;
+  const bool live = vec_site(a, parity, j, first);
+  if (live) {
+    Spinor<float> f;
+    SpinorIO<LQCD_F32>::load(PAR_PTR(a.r32, a.hbv), a.g.sstride, j, f);
+    convert(f, r);
+    red = site_norm2(r);
+  }
+  block_reduce_finalize<BLAS_BLOCK>(red, first, a.red, [&]() {
+    if (live) SpinorIO<RF>::store(PAR_PTR(a.rs, a.hbr), a.g.sstride, j, r);
+  });
 }
 
 // FP32 / 12-real copy of the FP64 links (rows 0 and 1, rounded once): the operator
@@ -208,15 +243,35 @@ __global__ void __launch_bounds__(BLAS_BLOCK) k_reconstruct_odd(Geom g, double* 
   SpinorIO<LQCD_F64>::store(xo, g.sstride, j, b);
 }
 
-// r_s = r - A x_s (FP32 arithmetic); |r_s|^2 -> beta, resume (FIN_MID)
+// Intermediate replacement: r_s = r - A x_s, r the residual of the last reliable
+// update and A x_s computed with FP32 arithmetic; |r_s|^2 -> beta, resume (FIN_MID).
+// The difference is taken in FP32: A x_s carries FP32 error already, and the
+// subtraction adds at most one rounding of r_s itself.
 template <int VF, int RF>
 __global__ void __launch_bounds__(BLAS_BLOCK) k_mid_residual(VecArgs a) {
+  using TV = typename PrecTraits<VF>::real;
   int parity;
   int64_t j, first;
   double red = 0.0;
-  if (vec_site(a, parity, j, first))
-    red = mid_residual_site<VF, RF>(a.g, j, PAR_PTR(a.r64, a.hb64), PAR_PTR(a.ax32, a.hbv), PAR_PTR(a.rs, a.hbr));
-  block_reduce_finalize<BLAS_BLOCK>(red, first, a.red);
+  Spinor<TV> rv;
+  const bool live = vec_site(a, parity, j, first);
+  if (live) {
+    Spinor<float> r, ax;
+    if (a.r32) {
+      SpinorIO<LQCD_F32>::load(PAR_PTR(a.r32, a.hbv), a.g.sstride, j, r);
+    } else {
+      Spinor<double> r64;
+      SpinorIO<LQCD_F64>::load(PAR_PTR(a.r64, a.hb64), a.g.sstride, j, r64);
+      convert(r64, r);
+    }
+    SpinorIO<LQCD_F32>::load(PAR_PTR(a.ax32, a.hbv), a.g.sstride, j, ax);
+#pragma unroll
+    for (int k = 0; k < 12; k++) rv.v[k] = mk((TV)(r.v[k].r - ax.v[k].r), (TV)(r.v[k].i - ax.v[k].i));
+    red = site_norm2(rv);
+  }
+  block_reduce_finalize<BLAS_BLOCK>(red, first, a.red, [&]() {
+    if (live) SpinorIO<RF>::store(PAR_PTR(a.rs, a.hbr), a.g.sstride, j, rv);
+  });
 }
 #undef PAR_PTR
 
@@ -372,7 +427,7 @@ struct Solver : CgEngine {
       af.b64 = b_full;
       af.red = rc_ss;
       af.red.result = w.bb;
-      k_b_minus<<<(unsigned)(2 * af.bpp), BLAS_BLOCK, 0, s>>>(af, nullptr, nullptr);
+      k_b_minus<LQCD_F64><<<(unsigned)(2 * af.bpp), BLAS_BLOCK, 0, s>>>(af, nullptr, nullptr);
       int st = after_launch("eo_solve: |b|^2");
       if (st) return st;
     }
@@ -384,21 +439,18 @@ struct Solver : CgEngine {
       const unsigned grid0 = (unsigned)(a.full ? 2 * a.bpp : a.bpp);
       VecArgs an = a;
       an.red = rc_ss;
-      k_b_minus<<<grid0, BLAS_BLOCK, 0, s>>>(an, nullptr, nullptr);
-      if ((st = after_launch("cgnr: |b|^2"))) return st;
       if (prm.sloppy_prec == LQCD_F64) {
+        k_b_minus<LQCD_F64><<<grid0, BLAS_BLOCK, 0, s>>>(an, nullptr, nullptr);
+        if ((st = after_launch("cgnr: |b|^2"))) return st;
         OpCtx c64{g, op64, gauge64};
         if ((st = op_apply(c64, w.ax64, a.b64, subset, 1, w.t1_64, w.t2_64, nullptr, nullptr, s))) return st;
         a.b64 = w.ax64;
       } else {
-        const unsigned grid = (unsigned)(a.full ? 2 * a.bpp : a.bpp);
-        k_copy_field<LQCD_F32, LQCD_F64><<<grid, BLAS_BLOCK, 0, s>>>(a, w.xs, a.b64);
-        if ((st = after_launch("cgnr: b to FP32"))) return st;
+        k_b_minus<LQCD_F32><<<grid0, BLAS_BLOCK, 0, s>>>(an, w.xs, nullptr);
+        if ((st = after_launch("cgnr: |b|^2, b to FP32"))) return st;
         OpCtx cm{g, opm, w.g32};
         if ((st = op_apply(cm, w.ax64, w.xs, subset, 1, w.t1_64, w.t2_64, nullptr, nullptr, s))) return st;
-        k_copy_field<LQCD_F64, LQCD_F32><<<grid, BLAS_BLOCK, 0, s>>>(a, w.mid64, w.ax64);
-        if ((st = after_launch("cgnr: M^dag b to FP64"))) return st;
-        a.b64 = w.mid64;
+        a.b32 = w.ax64;
       }
     }
     return launch_vec(VK_INIT, prm.sloppy_prec, a, s);
@@ -439,23 +491,22 @@ struct Solver : CgEngine {
     // CGNR: the FP64 residual of the system, s = b - M x and |s|^2, decides the exit;
     // r = M^dag s then only restarts the recurrence, in the inner arithmetic. The first
     // hop's H x stays in t1_64 (the odd half of an even-odd solve reuses it): the
-    // adjoint's temporaries are r64 (rewritten last) and t2_64.
+    // adjoint's temporaries are r64 (rewritten last) or mid64 (M x, used up) and t2_64.
     const unsigned grid = (unsigned)(a.full ? 2 * a.bpp : a.bpp);
     VecArgs an = a;
     an.red = rc_ss;
-    k_b_minus<<<grid, BLAS_BLOCK, 0, s>>>(an, w.mid64, w.mid64);
-    if ((st = after_launch("cgnr: b - M x"))) return st;
     a.red = rc_reliable;
     if (prm.sloppy_prec == LQCD_F64) {
+      k_b_minus<LQCD_F64><<<grid, BLAS_BLOCK, 0, s>>>(an, w.mid64, w.mid64);
+      if ((st = after_launch("cgnr: b - M x"))) return st;
       if ((st = op_apply(c64, w.ax64, w.mid64, subset, 1, w.r64, w.t2_64, nullptr, nullptr, s))) return st;
       a.b64 = nullptr;  // ax64 already holds the residual
       return launch_vec(VK_RESIDUAL, prm.sloppy_prec, a, s);
     }
-    k_copy_field<LQCD_F32, LQCD_F64><<<grid, BLAS_BLOCK, 0, s>>>(a, w.ax64, w.mid64);
-    if ((st = after_launch("cgnr: b - M x to FP32"))) return st;
+    k_b_minus<LQCD_F32><<<grid, BLAS_BLOCK, 0, s>>>(an, w.ax64, w.mid64);
+    if ((st = after_launch("cgnr: b - M x, to FP32"))) return st;
     OpCtx cm{g, opm, w.g32};
-    if ((st = op_apply(cm, w.mid64, w.ax64, subset, 1, w.r64, w.t2_64, nullptr, nullptr, s))) return st;
-    a.ax32 = w.mid64;
+    if ((st = op_apply(cm, a.r32, w.ax64, subset, 1, w.mid64, w.t2_64, nullptr, nullptr, s))) return st;
     return launch_vec(VK_RESIDUAL32, prm.sloppy_prec, a, s);
   }
 
@@ -584,6 +635,7 @@ static int cg_solve_impl(void* x, const void* b, const void* gauge, const void* 
   a.x64 = (double*)x;
   a.b64 = (const double*)b;
   a.r64 = S.w.r64;
+  a.r32 = normal && prm->sloppy_prec != LQCD_F64 ? S.w.r64 : nullptr;
   a.ax64 = S.w.ax64;
   a.xs = S.w.xs;
   a.rs = S.w.rs;
