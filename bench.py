@@ -661,9 +661,12 @@ def hop_roofline(L, F, lat, gsl, prec, flush, stream, vh, launches=40):
 
 HOP_SHAPE_MEANING = {0: "128 threads, one site per thread", 1: "128 threads, one site per thread, <= 72 registers",
                      2: "128 threads, one site per thread, spin components paired in packed FP32x2 arithmetic, "
-                        "<= 72 registers", 3: "128 threads, one site per thread, <= 102 registers",
-                     4: "128 threads, two sites per thread in packed FP32x2 arithmetic",
-                     5: "128 threads, one site per thread, links staged in shared memory when n5 >= 4",
+                        "<= 72 registers",
+                     3: "128 threads, one site per thread, links and neighbours staged in shared memory when n5 >= 4, "
+                        "spin-paired packed FP32x2 arithmetic, <= 64 registers",
+                     4: "as 3, <= 72 registers",
+                     5: "128 threads, one site per thread, links and neighbours staged in shared memory when n5 >= 4, "
+                        "<= 72 registers",
                      6: "128 threads, one site per thread, spin components paired in packed FP32x2 arithmetic",
                      7: "128 threads, one site per thread, <= 72 registers, neighbour spinors and links copied "
                         "asynchronously (cp.async) through a shared-memory ring",
@@ -1000,9 +1003,9 @@ def run_extras(L, F, flush, stream):
         tk, _ = _events_time(lambda: L.lqcd_force(Fo, g64, X, Y, lat, op, L.LQCD_FORCE_TA), stream, flush, reps=5)
         V = int(np.prod(dims))
         fbytes = V * (2 * 192 + 4 * 144 + 4 * 144)  # X, Y once per site, 4 links in, 4 force matrices out
-        # FP64 flop per link: 4 spin projections 48, two colour outer products 288, U A - B U^dag 432,
-        # boundary phase 18, traceless anti-Hermitian part 40
-        fflop = V * 4 * 826
+        # FP64 flop per link of the traceless-Hermitian kind: 4 spin projections 48, U on two pairs of half
+        # spinors 264, the Hermitian part of two outer products of them 240, phase, trace and scale 20
+        fflop = V * 4 * 572
         peak, _ = measured_peak()
         out[key] = {"ms_solve_and_force": round(ms, 3), "iterations": info.iterations,
                     "reliable_updates": info.reliable_updates,

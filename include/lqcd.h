@@ -383,10 +383,10 @@ int lqcd_batch_cg_solve(int n, const lqcd_batch_item* items, int recon, const lq
  *    launch-shape index of an FP32 / FP16 hop kernel (one site per thread
  *    with 0: 128 threads per block, registers as the compiler chooses; 1: 128
  *    threads and at least 7 resident blocks per SM; 2: as 6 with at least 7
- *    blocks per SM; 3: 128 threads and at least 5 blocks per SM; 4: 128 threads, two sites per
- *    thread in packed FP32x2 arithmetic, 3 blocks per SM; 5: 128 threads,
- *    one site per thread, at least 6 blocks per SM, the eight links of each 4D
- *    site loaded once into shared memory for its n5 threads when n5 >= 4;
+ *    blocks per SM; 5: 128 threads, one site per thread, at least 7 blocks per
+ *    SM, the eight links and neighbours of each 4D site staged once in shared
+ *    memory for its n5 threads when n5 >= 4 (shape 0 otherwise); 4 / 3: as 5
+ *    with the arithmetic of 6, at least 7 / 8 blocks per SM;
  *    6: 128 threads, one site per thread, the two spin components of each
  *    half spinor paired in packed FP32x2 arithmetic; 7 / 8: as 1 / 2 with
  *    each direction's neighbour spinor and link copied asynchronously into a

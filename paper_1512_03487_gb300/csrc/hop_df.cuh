@@ -12,7 +12,7 @@
 // neighbour data are copied into shared memory a phase ahead (cp.async, no register
 // holds them), which hides the loads at 16 warps per SM. M_hat (two hops) at 24^3 x
 // 48 with 18-real links on GB300: 593 -> 352 us against scalar instructions with the
-// loads where they are used; 22.2 -> 12.9 million warp instructions a hop, 64 % of
+// loads where they are used; 222 -> 129 million warp instructions a hop, 64 % of
 // the issue slots busy.
 #pragma once
 

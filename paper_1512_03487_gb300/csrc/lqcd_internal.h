@@ -36,7 +36,7 @@ constexpr int HOP_BLOCK = 128;
 // there; 110 without overlapped launches). 32^4 with 12 RHS, FP16: 1,434 (shape 0),
 // 1,411 (2), 1,239 (5), 1,217 (4), 1,186 (3); FP32: 1,729 (1), 1,606 (5), 1,681 (4),
 // 1,658 (3). Domain wall 16^4 x 16, FP32: 173 (2), 160 (5), 161 (4), 167 (3). Staging
-// takes 35 % of the instructions out (44.5 -> 27.8 million warp instructions a hop for
+// takes 35 % of the instructions out (445 -> 278 million warp instructions a hop for
 // 12 RHS); what is left waits for loads, so that resident warps pay even at the price
 // of some spilled registers (5, 6, 7, 8 blocks per SM, FP16: 1,321, 1,255, 1,219, 1,186).
 // Shape 0 is the default; the tuner times all of them per key.
