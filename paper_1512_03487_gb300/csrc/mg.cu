@@ -245,7 +245,10 @@ __global__ void __launch_bounds__(MG_BLOCK) k_block_orth(void* vecs, MGGeom m) {
 // Sums of the restriction: FP32 fields add theirs up as double-float pairs, FP64 fields
 // in FP64. FP64 additions run at 1/64 of the FP32 rate (they were 71 % of the FP64
 // pipe's time when FP32 terms were summed in FP64), and the 48 bits of a pair are far
-// below the FP32 rounding of the terms and of the result.
+// below the FP32 rounding of the terms and of the result. A pair has FP32's range, and
+// an infinite or NaN term or a partial sum beyond 2^128 leaves it not finite for good
+// (its conversion to FP64 works on the bits and is for finite ones): a warp that ends
+// with such a pair adds its FP32 terms up again in FP64, which carries those values.
 template <typename T> struct SumOf;
 template <> struct SumOf<float> { using type = dfl; };
 template <> struct SumOf<double> { using type = double; };
@@ -261,6 +264,8 @@ __device__ __forceinline__ dfl add_term(dfl s, float v) {
   return fast_two_sum(h, e + s.lo);
 }
 __device__ __forceinline__ double add_term(double s, double v) { return s + v; }
+__device__ __forceinline__ bool sum_finite(dfl v) { return fabsf(v.hi) < INFINITY; }
+__device__ __forceinline__ bool sum_finite(double) { return true; }  // FP64 sums are never made again
 
 // c(X)[(s, k)] = sum_{x in X} P_k(x)|_s^dag psi(x)|_s. One thread per fine site, 256
 // sites per block (one aggregate of 4^4 or 16 of 2^4), all vectors: psi is read once
@@ -314,18 +319,23 @@ __global__ void __launch_bounds__(RS_BLOCK, P == LQCD_F32 ? 4 : 1) k_restrict(vo
       }
     }
     __syncthreads();
-    S s = S(0);
+    const auto total = [&](auto s) {
 #pragma unroll
-    for (int i = 0; i < 16; i++) s = add_term(s, buf[val * PITCH + start + i * stride]);
-    if (BUFS == 1) __syncthreads();
-    if (B == 4) {
+      for (int i = 0; i < 16; i++) s = add_term(s, buf[val * PITCH + start + i * stride]);
+      if (BUFS == 1) __syncthreads();
+      if (B == 4) {
 #pragma unroll
-      for (int o = 8; o > 0; o >>= 1) s = s + xor_lanes(s, o);
-    }
+        for (int o = 8; o > 0; o >>= 1) s = s + xor_lanes(s, o);
+      }
+      return s;
+    };
+    const S s = total(S(0));
+    double sum = sum_value(s);
+    if (P == LQCD_F32 && __any_sync(0xffffffffu, !sum_finite(s))) sum = total(0.0);
     // value: vector k0 + val / 4, chirality (val / 2) % 2, real or imaginary part
     const int k = k0 + (val >> 2);
     if (act && k < m.nv && (B == 2 || (tid & 15) == 0))
-      out[(agg * m.nc + ((val >> 1) & 1) * m.nv + k) * 2 + (val & 1)] = (T)sum_value(s);
+      out[(agg * m.nc + ((val >> 1) & 1) * m.nv + k) * 2 + (val & 1)] = (T)sum;
   }
 }
 
@@ -381,38 +391,25 @@ __device__ __forceinline__ int64_t coarse_nb(const MGGeom& m, int64_t X, int d) 
 // lengths that are not a multiple of four pieces, or long. 2,592 sites of 24 x 24
 // blocks in FP32 on GB300: 55 -> 30 us (before: one warp per row, divisions per product).
 constexpr int CA_LANES = 4;
-template <typename T, int NP>
-__global__ void __launch_bounds__(MG_BLOCK) k_coarse_apply(cpx<T>* out, const cpx<T>* in, const cpx<T>* Y, MGGeom m) {
-  constexpr int PER = 16 / (int)sizeof(cpx<T>);  // complex values per 16-byte piece
-  struct alignas(16) Piece { cpx<T> v[PER]; };
-  using S = typename SumOf<T>::type;
-  const int nc = m.nc, rows = 32 / CA_LANES, groups = (nc + rows - 1) / rows;
-  const int wid = (int)(((int64_t)blockIdx.x * MG_BLOCK + threadIdx.x) >> 5);  // below Vc groups < 2^31
-  const int lane = threadIdx.x & 31;
-  if (wid >= m.Vc * groups) return;  // whole warps exit together
-  const int X = wid / groups;
-  const int i = (wid - X * groups) * rows + lane / CA_LANES, l = lane % CA_LANES;
-  int nb_l = X;  // lanes 1..8 find the stencil's neighbours (32-bit index arithmetic)
-  {
-    const int mu = (lane - 1) >> 1, stx = m.cX, sty = stx * m.cY, stz = sty * m.cZ;
-    const int L = mu == 0 ? m.cX : mu == 1 ? m.cY : mu == 2 ? m.cZ : m.cT;
-    const int st = mu == 0 ? 1 : mu == 1 ? stx : mu == 2 ? sty : stz;
-    const int at = X / st % L;
-    if (lane > 0 && lane < 9)
-      nb_l += (lane & 1) ? (at == L - 1 ? -(L - 1) * st : st) : (at == 0 ? (L - 1) * st : -st);
-  }
+template <typename T> struct alignas(16) Piece {
+  cpx<T> v[16 / sizeof(cpx<T>)];
+};
+
+// Lane l's share of a row's sum over the nine blocks, then the sum over the row's lanes: a
+// block's products in T, their sum in S. y: the lane's first piece of block 0; every
+// lane of the warp must call it. BLOCKS: blocks whose loads are in flight together.
+template <typename S, int NP, int BLOCKS, typename T>
+__device__ __forceinline__ void coarse_row(const Piece<T>* y, int64_t ystep, const cpx<T>* in, int nc, int nb_l, int l,
+                                           S& sr, S& si) {
+  constexpr int PER = 16 / (int)sizeof(cpx<T>);
   const int pieces = nc / PER;
-  const int64_t block = (int64_t)nc * nc;
-  const Piece* y = reinterpret_cast<const Piece*>(Y + X * block + (int64_t)(i < nc ? i : 0) * nc) + l;
-  const int64_t ystep = m.Vc * block / PER;
-  // a block's products in T, the sum over the blocks and lanes as in the restriction
-  S sr = S(0), si = S(0);
-#pragma unroll
+  sr = si = S(0);
+#pragma unroll BLOCKS
   for (int d = 0; d < 9; d++) {
     const int Xn = __shfl_sync(0xffffffffu, nb_l, d);
-    const Piece* v = reinterpret_cast<const Piece*>(in + (int64_t)Xn * nc) + l;
+    const Piece<T>* v = reinterpret_cast<const Piece<T>*>(in + (int64_t)Xn * nc) + l;
     T r = T(0), q = T(0);
-    auto add = [&](const Piece& w, const Piece& x) {
+    auto add = [&](const Piece<T>& w, const Piece<T>& x) {
 #pragma unroll
       for (int e = 0; e < PER; e++) {
         r = fma(w.v[e].r, x.v[e].r, fma(-w.v[e].i, x.v[e].i, r));
@@ -434,7 +431,35 @@ __global__ void __launch_bounds__(MG_BLOCK) k_coarse_apply(cpx<T>* out, const cp
     sr = sr + xor_lanes(sr, o);
     si = si + xor_lanes(si, o);
   }
-  if (l == 0 && i < nc) out[(int64_t)X * nc + i] = mk((T)sum_value(sr), (T)sum_value(si));
+}
+
+template <typename T, int NP>
+__global__ void __launch_bounds__(MG_BLOCK) k_coarse_apply(cpx<T>* out, const cpx<T>* in, const cpx<T>* Y, MGGeom m) {
+  using S = typename SumOf<T>::type;
+  const int nc = m.nc, rows = 32 / CA_LANES, groups = (nc + rows - 1) / rows;
+  const int wid = (int)(((int64_t)blockIdx.x * MG_BLOCK + threadIdx.x) >> 5);  // below Vc groups < 2^31
+  const int lane = threadIdx.x & 31;
+  if (wid >= m.Vc * groups) return;  // whole warps exit together
+  const int X = wid / groups;
+  const int i = (wid - X * groups) * rows + lane / CA_LANES, l = lane % CA_LANES;
+  int nb_l = X;  // lanes 1..8 find the stencil's neighbours (32-bit index arithmetic)
+  {
+    const int mu = (lane - 1) >> 1, stx = m.cX, sty = stx * m.cY, stz = sty * m.cZ;
+    const int L = mu == 0 ? m.cX : mu == 1 ? m.cY : mu == 2 ? m.cZ : m.cT;
+    const int st = mu == 0 ? 1 : mu == 1 ? stx : mu == 2 ? sty : stz;
+    const int at = X / st % L;
+    if (lane > 0 && lane < 9)
+      nb_l += (lane & 1) ? (at == L - 1 ? -(L - 1) * st : st) : (at == 0 ? (L - 1) * st : -st);
+  }
+  const int64_t block = (int64_t)nc * nc;
+  const Piece<T>* y = reinterpret_cast<const Piece<T>*>(Y + X * block + (int64_t)(i < nc ? i : 0) * nc) + l;
+  const int64_t ystep = m.Vc * block / (16 / (int)sizeof(cpx<T>));
+  S sr, si;
+  coarse_row<S, NP, 9>(y, ystep, in, nc, nb_l, l, sr, si);
+  double re = sum_value(sr), im = sum_value(si);
+  if (sizeof(T) == 4 && __any_sync(0xffffffffu, !sum_finite(sr) || !sum_finite(si)))
+    coarse_row<double, 0, 1>(y, ystep, in, nc, nb_l, l, re, im);
+  if (l == 0 && i < nc) out[(int64_t)X * nc + i] = mk((T)re, (T)im);
 }
 
 // The adjoint, out(X)_i = sum_d sum_j conj(Y_{-d}(X + d)_ji) in(X + d)_j, from the
