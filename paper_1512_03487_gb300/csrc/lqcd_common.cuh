@@ -53,12 +53,18 @@ inline cudaError_t launch_overlapped(void (*kernel)(Arg), unsigned grid, unsigne
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, arg);
 }
-// Lets the next kernel on the stream start and waits until the ones before have
+// Lets the next kernel on the stream start (EARLY) and waits until the ones before have
 // finished and their writes are visible. Every thread of every block calls it, also
 // one that returns at once: a kernel that ended without waiting would release its
 // successor while its predecessor still runs.
-__device__ __forceinline__ void overlap_launch() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+// A kernel that asks for the largest shared-memory carveout does not let its successor
+// start early (it may still start early itself): the successor would take the SMs as
+// they are, with the small L1 that is left, and so would all that follow it in a chain
+// of overlapping launches. M_hat^dag M_hat at 24^3 x 48, FP32, the first hop in the
+// ring shape and three plain ones: 198 us with its early start, 143 without, 143 for
+// four plain hops; four ring hops 142 either way (16^3 x 32: 42 with, 29 without).
+template <bool EARLY> __device__ __forceinline__ void overlap_launch() {
+  if constexpr (EARLY) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
