@@ -588,6 +588,7 @@ int lqcd_batch_cg_solve(int n, const lqcd_batch_item* items, int recon, const lq
   }
   S.set_tile(tile);
   S.grid = (unsigned)std::min<int64_t>(std::min<int64_t>((int64_t)bps * sms, S.total_tiles), MAX_GRID);
+  S.blocks = S.grid;
 
   std::vector<unsigned char> key;
   int dev = 0;

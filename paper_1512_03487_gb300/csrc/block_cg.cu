@@ -788,6 +788,7 @@ int lqcd_block_cg_solve(void* x, const void* b, const void* gauge, const void* g
     return finish(fail(LQCD_ERR_WORKSPACE, "block cg: workspace %zu < %zu bytes", workspace_bytes, S.w.total));
   S.N = S.g.n5;
   S.nsys = S.N;
+  S.blocks = (S.g.nsites + HOP_BLOCK - 1) / HOP_BLOCK;
   S.ctrl = S.w.ctrl;
   S.sys = S.w.sys;
   S.sloppy = prm->sloppy_prec;

@@ -611,6 +611,7 @@ static int cg_solve_impl(void* x, const void* b, const void* gauge, const void* 
     return finish(fail(LQCD_ERR_WORKSPACE, "cg: workspace %zu < %zu bytes", workspace_bytes, S.w.total));
   S.ctrl = S.w.ctrl;
   S.sys = S.w.sys;
+  S.blocks = (S.g.nsites + HOP_BLOCK - 1) / HOP_BLOCK * (subset == LQCD_FULL ? 2 : 1);
   S.op64 = *op;
   // mixed Wilson solves may run the reliable updates' FP64-field operator in double-float arithmetic
   if (update_df(*op, *prm, lat->n5)) S.op64.prec = LQCD_F64_DF;

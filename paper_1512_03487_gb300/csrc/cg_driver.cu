@@ -12,10 +12,7 @@
 //
 // An iteration that requests an update pauses the solve (active = 0), so that the
 // rest of the body's kernels return at once, and the branch resumes it. U, the
-// iterations per body, is the largest divisor of check_interval up to UNROLL: the
-// WHILE and IF nodes and the control kernel cost about 20 us per body on GB300
-// (iteration at 24^3 x 48, FP16, three levels: 158 us with U = 1, 143 with 8;
-// 12^3 x 24, FP32: 39 us, 32), a skipped iteration about 10 us.
+// iterations per body, is chosen per solve (iterations_per_body).
 //
 // The WHILE and IF conditions are set on the device (cudaGraphSetConditional)
 // by a one-thread control kernel and by the finaliser of the update kernel,
@@ -26,6 +23,7 @@
 //
 // With use_graph = 0 the same kernels are launched directly and a requested
 // reliable update pauses the chunk for the host instead.
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 
@@ -50,10 +48,30 @@ __global__ void k_loop_control(Control* c, int maxiter, cudaGraphConditionalHand
   cudaGraphSetConditional(h_loop, go ? 1u : 0u);
 }
 
-constexpr int UNROLL = 8;
-static int unroll_of(int chunk) {
-  int u = UNROLL;
-  while (chunk % u) u--;
+// U, the iterations per body of the graph. The WHILE and IF nodes and the control
+// kernel cost 7 to 14 us per body on GB300; an iteration launched behind a pause costs 6 us,
+// and 5 us more per 1,000 blocks of a hop (which all start and return). So U must not
+// pass the distance between pauses by much, and an update is due whenever the
+// residual has fallen by delta (delta_mid: a replacement), on well-conditioned
+// links every 2 iterations at 0.3 and every 3 at 0.1 (Haar-distributed links fall by 2.7 per
+// iteration; others take longer, and lose less). Whole even-odd solves in ms, U = 1 / 2 / 4 / 8:
+//   12^3 x 24 FP32, delta 0.9         3.05  3.17  3.43    -     (an update in each of 23 iterations)
+//                   delta 0.3         2.16  2.01  2.12  2.44    (12 updates)
+//                   delta 0.1         1.77  1.75  1.72  2.00    (8)
+//                   delta 0.01        1.56  1.45  1.45  1.45    (5)
+//                   delta 3e-6        1.31  1.16  1.13  1.14    (2)
+//   24^3 x 48 FP32, delta 0.3        22.36 21.95 21.92 23.20    (17 of 60)
+//             FP16, 0.003 and 3e-6   11.29 11.20 11.03 11.23    (5 pauses of 61)
+//             FP32, delta 3e-6       14.33 13.89 13.77 13.71    (2)
+//   two columns, delta 0.1           35.03 34.91 34.92    -     (5,184 blocks)
+//   four columns, delta 0.1          60.86 60.97 61.22    -     (10,368 blocks)
+//   32^4, 12 columns, FP16           91.57 91.91 94.33 95.28    (49,152 blocks, 5 pauses of 24)
+constexpr int64_t MAX_SKIPPED_BLOCKS = 6144;
+static int iterations_per_body(const CgEngine& E, const lqcd_solver_params& prm, int chunk) {
+  const double delta = prm.sloppy_prec == LQCD_F64 ? 0.0  // paused at the end only
+                       : E.has_mid() ? std::max(prm.delta, prm.delta_mid) : prm.delta;
+  int u = E.blocks > MAX_SKIPPED_BLOCKS || delta > 0.3 ? 1 : delta > 0.1 ? 2 : 4;
+  while (chunk % u) u--;  // a chunk is a whole number of bodies
   return u;
 }
 
@@ -101,7 +119,7 @@ struct Capture {
     if (e_ != cudaSuccess) return cuda_fail(e_, what); \
   } while (0)
 
-static int build_graph(CgEngine& E, int chunk, int maxiter, GraphEntry* out) {
+static int build_graph(CgEngine& E, int chunk, int unroll, int maxiter, GraphEntry* out) {
   Capture cap;
   LQCD_TRY_CUDA(cudaStreamCreateWithFlags(&cap.s, cudaStreamNonBlocking), "cg graph: stream");
   cudaGraph_t outer = nullptr;
@@ -144,7 +162,6 @@ static int build_graph(CgEngine& E, int chunk, int maxiter, GraphEntry* out) {
                   "cg graph: replacement handle");
 
   // body: the iterations
-  const int unroll = unroll_of(chunk);
   LQCD_TRY_CUDA(cudaStreamBeginCaptureToGraph(cap.s, body, nullptr, nullptr, 0, mode), "cg graph: capture");
   uint64_t c0 = g_captured_launches;
   for (int u = 0; u < unroll && !st; u++)
@@ -210,8 +227,8 @@ static int build_graph(CgEngine& E, int chunk, int maxiter, GraphEntry* out) {
   return LQCD_OK;
 }
 
-static int cached_graph(CgEngine& E, const std::vector<unsigned char>& key, int chunk, int maxiter,
-                        GraphEntry* out) {
+static int cached_graph(CgEngine& E, const std::vector<unsigned char>& key, int chunk, int unroll,
+                        int maxiter, GraphEntry* out) {
   std::lock_guard<std::mutex> lock(g_graph_mutex);
   for (auto& e : g_graphs) {
     if (e.key == key) {
@@ -223,7 +240,7 @@ static int cached_graph(CgEngine& E, const std::vector<unsigned char>& key, int 
   GraphEntry ne;
   ne.key = key;
   ne.exec = nullptr;
-  int st = build_graph(E, chunk, maxiter, &ne);
+  int st = build_graph(E, chunk, unroll, maxiter, &ne);
   if (st) {
     if (ne.exec) cudaGraphExecDestroy(ne.exec);
     return st;
@@ -248,14 +265,16 @@ static int read_ctrl(const Control* d, Control* h, cudaStream_t s) {
   return LQCD_OK;
 }
 
-int run_cg(CgEngine& E, const lqcd_solver_params& prm, const std::vector<unsigned char>& key, cudaStream_t s,
+int run_cg(CgEngine& E, const lqcd_solver_params& prm, std::vector<unsigned char> key, cudaStream_t s,
            std::chrono::steady_clock::time_point t0, Control* ctrl) {
   int st = E.init(s);
   if (st) return st;
   const int chunk = prm.check_interval > 0 ? prm.check_interval : 16;
+  const int unroll = iterations_per_body(E, prm, chunk);
+  key_append(key, unroll);
   GraphEntry ge;
   ge.exec = nullptr;
-  if (prm.use_graph && (st = cached_graph(E, key, chunk, prm.maxiter, &ge))) return st;
+  if (prm.use_graph && (st = cached_graph(E, key, chunk, unroll, prm.maxiter, &ge))) return st;
   auto timed_out = [&]() {
     if (prm.timeout_ms <= 0) return false;
     const double el = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
@@ -273,7 +292,7 @@ int run_cg(CgEngine& E, const lqcd_solver_params& prm, const std::vector<unsigne
       cudaError_t e = cudaGraphLaunch(ge.exec, s);
       if (e != cudaSuccess) return cuda_fail(e, "cg: graph launch");
       if ((st = read_ctrl(E.ctrl, ctrl, s))) return st;
-      const uint64_t bodies = (uint64_t)((chunk - ctrl->chunk_left) / unroll_of(chunk));
+      const uint64_t bodies = (uint64_t)((chunk - ctrl->chunk_left) / unroll);
       const uint64_t rels = (uint64_t)(ctrl->n_reliable - before.n_reliable);
       const uint64_t mids = (uint64_t)(ctrl->n_mid - before.n_mid);
       count_launches(1 + bodies * ge.body_kernels + rels * ge.reliable_kernels + mids * ge.mid_kernels);

@@ -14,6 +14,7 @@ struct CgEngine {
   Control* ctrl = nullptr;
   SysState* sys = nullptr;
   int nsys = 0;
+  int64_t blocks = 0;  // thread blocks of one of an iteration's hops
   virtual ~CgEngine() {}
   // r = b, x = 0, p = b; |b|^2 per system -> initial state (FIN_INIT)
   virtual int init(cudaStream_t s) = 0;
@@ -33,10 +34,11 @@ struct CgEngine {
 };
 
 // Runs a solve with engine E. `key` identifies everything the captured graph
-// bakes in (pointers, shapes, formats, chunk length, iteration cap); graphs
-// are cached across calls under it. On return *ctrl holds the final control
+// bakes in (pointers, shapes, formats, chunk length, iteration cap), but for the
+// iterations per graph body, which the driver chooses and adds; graphs are
+// cached across calls under it. On return *ctrl holds the final control
 // block.
-int run_cg(CgEngine& E, const lqcd_solver_params& prm, const std::vector<unsigned char>& key, cudaStream_t s,
+int run_cg(CgEngine& E, const lqcd_solver_params& prm, std::vector<unsigned char> key, cudaStream_t s,
            std::chrono::steady_clock::time_point t0, Control* ctrl);
 
 // Kernel launches are counted when they run: a thread capturing a graph
