@@ -403,8 +403,10 @@ int lqcd_batch_cg_solve(int n, const lqcd_batch_item* items, int recon, const lq
  *    per configuration in a tuning pass on their own workspace before the
  *    first iteration. Untimed keys use shape 0.
  * lqcd_tune_save writes the table to a text file (one "value<TAB>key" line
- * per entry); lqcd_tune_load reads one back (its entries replace current
- * ones; loaded hop keys are never re-timed); lqcd_tune_entries counts the
+ * per entry; a hop's line ends in "<TAB>shapes=V", V the version of the list
+ * of launch shapes); lqcd_tune_load reads one back (its entries replace current
+ * ones; loaded hop keys are never re-timed; a hop's line with another V is
+ * skipped, one without V is taken as it is); lqcd_tune_entries counts the
  * entries; lqcd_tune_get returns the value stored for key, or -1;
  * lqcd_tune_clear forgets every entry (hops are timed again on next use);
  * lqcd_tune_set_enabled(0) stops all timing (untimed keys then keep their

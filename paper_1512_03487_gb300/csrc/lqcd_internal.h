@@ -43,6 +43,8 @@ constexpr int HOP_BLOCK = 128;
 #define LQCD_HOP_SHAPES(X) X(0, 128, 1, 0) X(1, 128, 1, 7) X(2, 128, -2, 7) X(3, 128, -5, 8) X(4, 128, -5, 7) \
   X(5, 128, -1, 7) X(6, 128, -2, 0) X(7, 128, -3, 7) X(8, 128, -4, 7)
 constexpr int HOP_SHAPES = 9;
+// Raised whenever an index comes to mean another kernel: saved tables carry it.
+constexpr int HOP_SHAPES_VERSION = 2;
 // Whether shape i differs from shape 0 for n5 slices (the tuner skips it otherwise).
 inline bool hop_shape_applies(int i, int n5) { return (i != 3 && i != 4 && i != 5) || n5 >= STAGE_MIN_N5; }
 // The shape used when the table holds no choice for a hop.

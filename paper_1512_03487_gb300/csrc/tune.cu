@@ -35,6 +35,14 @@ void tune_store(const std::string& key, int value) {
   g_tune_version++;
 }
 
+// A hop's choice is an index into LQCD_HOP_SHAPES, so its line in a saved table also
+// names the list's version: under another list the number means another kernel.
+static bool is_hop_key(const std::string& key) { return key.compare(0, 4, "hop ") == 0; }
+static const std::string& shapes_tag() {
+  static const std::string tag = "shapes=" + std::to_string(HOP_SHAPES_VERSION);
+  return tag;
+}
+
 }  // namespace lqcd
 
 using namespace lqcd;
@@ -46,7 +54,9 @@ int lqcd_tune_save(const char* path) {
   FILE* f = fopen(path, "w");
   if (!f) return fail(LQCD_ERR_ARG, "lqcd_tune_save: cannot open %s", path);
   std::lock_guard<std::mutex> lock(g_tune_mutex);
-  for (auto& kv : g_tune) fprintf(f, "%d\t%s\n", kv.second, kv.first.c_str());
+  for (auto& kv : g_tune)
+    fprintf(f, "%d\t%s%s%s\n", kv.second, kv.first.c_str(), is_hop_key(kv.first) ? "\t" : "",
+            is_hop_key(kv.first) ? shapes_tag().c_str() : "");
   fclose(f);
   return LQCD_OK;
 }
@@ -66,6 +76,11 @@ int lqcd_tune_load(const char* path) {
     if (end == line || *end != 0) continue;
     std::string k(tab + 1);
     while (!k.empty() && (k.back() == '\n' || k.back() == '\r')) k.pop_back();
+    if (is_hop_key(k) && k.find('\t') != std::string::npos) {
+      const size_t end_of_key = k.find('\t');
+      if (k.compare(end_of_key + 1, std::string::npos, shapes_tag()) != 0) continue;  // timed again on next use
+      k.resize(end_of_key);
+    }
     if (k.empty() || v < 0 || v > 64) continue;
     g_tune[k] = (int)v;
   }
