@@ -183,7 +183,6 @@ __device__ __forceinline__ void link_mul_dag(const Link<T>& u, const Half<T>& h,
 template <typename T> __device__ __forceinline__ T bc_phase(const Geom& g, int mu);
 template <> __device__ __forceinline__ double bc_phase<double>(const Geom& g, int mu) { return g.bcd[mu]; }
 template <> __device__ __forceinline__ float bc_phase<float>(const Geom& g, int mu) { return g.bcf[mu]; }
-template <> __device__ __forceinline__ dfl bc_phase<dfl>(const Geom& g, int mu) { return dfl(g.bcf[mu], 0.f); }
 
 // FP32 a + c and a - c for a the low (H = 0) or high (H = 1) FP16 half of the
 // word w (add / sub with an f16 and an f32 operand, sm_100 and later): the
@@ -412,37 +411,36 @@ __device__ __forceinline__ void hop_acc(const Geom& g, const void* gauge, const 
                                         Spinor<typename PrecTraits<P>::real>& acc, unsigned char* ring = nullptr) {
   if constexpr (P == LQCD_F64_DF) {
     hop_acc_df<R, DAG, AS, BLOCK>(g, gauge, in, parity, j, acc, ring);
-    return;
   } else if constexpr (AS) {
     hop_acc_async<P, R, DAG, SP, BLOCK>(g, gauge, in, parity, j, acc, ring);
-    return;
-  }
-  const int64_t n5 = g.n5;
-  int64_t cb, i5;
-  if (n5 == 1) {
-    cb = j;
-    i5 = 0;
   } else {
-    cb = fdiv((uint32_t)j, g.fn5);
-    i5 = j - cb * n5;
+    const int64_t n5 = g.n5;
+    int64_t cb, i5;
+    if (n5 == 1) {
+      cb = j;
+      i5 = 0;
+    } else {
+      cb = fdiv((uint32_t)j, g.fn5);
+      i5 = j - cb * n5;
+    }
+    const Coord x = cb_to_coord(g, cb, parity);
+    if constexpr (SP) {
+      static_assert(P == LQCD_F32 || P == LQCD_F16, "spin-paired hop: FP32 / FP16 storage");
+      SPAcc a;
+      sp_zero(a);
+      hop_dir_sp<0, P, R, DAG>(a, g, gauge, x, cb, i5, parity, in);
+      hop_dir_sp<1, P, R, DAG>(a, g, gauge, x, cb, i5, parity, in);
+      hop_dir_sp<2, P, R, DAG>(a, g, gauge, x, cb, i5, parity, in);
+      hop_dir_sp<3, P, R, DAG>(a, g, gauge, x, cb, i5, parity, in);
+      sp_unpack(a, acc);
+    } else {
+      zero(acc);
+      hop_dir<0, P, R, DAG, GP>(acc, g, gauge, x, cb, i5, parity, in);
+      hop_dir<1, P, R, DAG, GP>(acc, g, gauge, x, cb, i5, parity, in);
+      hop_dir<2, P, R, DAG, GP>(acc, g, gauge, x, cb, i5, parity, in);
+      hop_dir<3, P, R, DAG, GP>(acc, g, gauge, x, cb, i5, parity, in);
+    }
   }
-  const Coord x = cb_to_coord(g, cb, parity);
-  if constexpr (SP) {
-    static_assert(P == LQCD_F32 || P == LQCD_F16, "spin-paired hop: FP32 / FP16 storage");
-    SPAcc a;
-    sp_zero(a);
-    hop_dir_sp<0, P, R, DAG>(a, g, gauge, x, cb, i5, parity, in);
-    hop_dir_sp<1, P, R, DAG>(a, g, gauge, x, cb, i5, parity, in);
-    hop_dir_sp<2, P, R, DAG>(a, g, gauge, x, cb, i5, parity, in);
-    hop_dir_sp<3, P, R, DAG>(a, g, gauge, x, cb, i5, parity, in);
-    sp_unpack(a, acc);
-    return;
-  }
-  zero(acc);
-  hop_dir<0, P, R, DAG, GP>(acc, g, gauge, x, cb, i5, parity, in);
-  hop_dir<1, P, R, DAG, GP>(acc, g, gauge, x, cb, i5, parity, in);
-  hop_dir<2, P, R, DAG, GP>(acc, g, gauge, x, cb, i5, parity, in);
-  hop_dir<3, P, R, DAG, GP>(acc, g, gauge, x, cb, i5, parity, in);
 }
 
 // The epilogue at output site j of the hop result acc = H in (see EpiCoef).

@@ -1,8 +1,8 @@
 // The hop in double-float arithmetic on FP64 fields (LQCD_F64_DF), with the two
 // spin components of each half spinor in packed FP32x2 instructions.
 //
-// Every operation is the scalar double-float operation of df.cuh, two at a time, so
-// the results are bit-identical to it; the kernel is bound by instructions (about
+// Every operation is the scalar double-float operation of df.cuh, two at a time, with the
+// same roundings; the kernel is bound by instructions (about
 // 1,800 FP32 operations and 250 integer ones of the splits per direction and thread).
 // Three things keep it fast. (1) A pair (spin 0, spin 1) shares every packed
 // instruction (add / mul / fma.rn.f32x2; negated and broadcast operands cost

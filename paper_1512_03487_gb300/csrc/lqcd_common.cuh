@@ -260,23 +260,6 @@ template <> struct SpinorIO<LQCD_F16> {
       }
     }
   }
-  // Components without the site norm (returned separately), so that a caller
-  // can apply the norm after a linear map that shrinks the data (spin projection).
-  static __device__ __forceinline__ void load_unscaled(const void* base, int64_t stride, int64_t j, Spinor<T>& s,
-                                                       float& nrm) {
-    const uint4* b = reinterpret_cast<const uint4*>(base);
-    nrm = norm_ptr(base, stride)[j];
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-      uint4 w = b[c * stride + j];
-      unsigned int words[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-      for (int q = 0; q < 4; q++) {
-        float2 f = __half22float2(*reinterpret_cast<__half2*>(&words[q]));
-        s.v[4 * c + q] = mk(f.x, f.y);
-      }
-    }
-  }
   static __device__ __forceinline__ void store(void* base, int64_t stride, int64_t j, const Spinor<T>& s) {
     float m = 0.f;
 #pragma unroll
@@ -338,25 +321,6 @@ template <> struct LinkIO<LQCD_F64, 12> {
     const double2* b = reinterpret_cast<const double2*>(g) + (int64_t)blk * NCHUNK * gs + cb;
 #pragma unroll
     for (int c = 0; c < 6; c++) { double2 w = b[c * gs]; u.v[c] = mk(w.x, w.y); }
-    rebuild_row2(u);
-  }
-};
-template <> struct LinkIO<LQCD_F64_DF, 18> {
-  using T = dfl;
-  static constexpr int NCHUNK = 9;
-  static __device__ __forceinline__ void load(const void* g, int64_t gs, int blk, int64_t cb, Link<T>& u) {
-    const double2* b = reinterpret_cast<const double2*>(g) + (int64_t)blk * NCHUNK * gs + cb;
-#pragma unroll
-    for (int c = 0; c < 9; c++) { double2 w = b[c * gs]; u.v[c] = mk(df_split(w.x), df_split(w.y)); }
-  }
-};
-template <> struct LinkIO<LQCD_F64_DF, 12> {
-  using T = dfl;
-  static constexpr int NCHUNK = 6;
-  static __device__ __forceinline__ void load(const void* g, int64_t gs, int blk, int64_t cb, Link<T>& u) {
-    const double2* b = reinterpret_cast<const double2*>(g) + (int64_t)blk * NCHUNK * gs + cb;
-#pragma unroll
-    for (int c = 0; c < 6; c++) { double2 w = b[c * gs]; u.v[c] = mk(df_split(w.x), df_split(w.y)); }
     rebuild_row2(u);
   }
 };
