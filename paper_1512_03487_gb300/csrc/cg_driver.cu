@@ -66,11 +66,12 @@ __global__ void k_loop_control(Control* c, int maxiter, cudaGraphConditionalHand
 //   two columns, delta 0.1           35.03 34.91 34.92    -     (5,184 blocks)
 //   four columns, delta 0.1          60.86 60.97 61.22    -     (10,368 blocks)
 //   32^4, 12 columns, FP16           91.57 91.91 94.33 95.28    (49,152 blocks, 5 pauses of 24)
+//   16^4 FP32, delta 1e-5 (HMC trajectory) -    -   88.15 86.91   (2 of 93 in each solve)
 constexpr int64_t MAX_SKIPPED_BLOCKS = 6144;
 static int iterations_per_body(const CgEngine& E, const lqcd_solver_params& prm, int chunk) {
   const double delta = prm.sloppy_prec == LQCD_F64 ? 0.0  // paused at the end only
                        : E.has_mid() ? std::max(prm.delta, prm.delta_mid) : prm.delta;
-  int u = E.blocks > MAX_SKIPPED_BLOCKS || delta > 0.3 ? 1 : delta > 0.1 ? 2 : 4;
+  int u = E.blocks > MAX_SKIPPED_BLOCKS || delta > 0.3 ? 1 : delta > 0.1 ? 2 : delta > 1e-4 ? 4 : 8;
   while (chunk % u) u--;  // a chunk is a whole number of bodies
   return u;
 }
