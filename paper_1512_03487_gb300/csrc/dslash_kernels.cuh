@@ -630,7 +630,7 @@ template <int P, int R, bool DAG, int EPI, int RED, int BLOCK, bool GP, bool LS 
           bool AS = false>
 __device__ __forceinline__ void hop_body(const HopArgs& A) {
   using T = typename PrecTraits<P>::real;
-  overlap_launch<!AS>();  // AS: the ring's shared-memory carveout
+  overlap_wait();
   if (gate_closed(A.gate)) return;
   int parity = A.out_parity;
   int blk = blockIdx.x;

@@ -27,14 +27,20 @@ int after_launch(const char* what);
 
 inline int64_t round_up(int64_t a, int64_t b) { return (a + b - 1) / b * b; }
 
-// Launches kernel so that it may start while the kernel before it on the stream still
-// runs (programmatic dependent launch): its blocks take the SMs that the other's last
-// blocks leave idle and do their index arithmetic there. The kernel calls
-// overlap_launch() before it touches memory. A predecessor that does not take part
-// is waited for as usual. Back to back on one stream it gains 7-8 % at 24^3 x 48 and
-// below (FP16 M^dag M 110 -> 102 us, 8^4 FP32 24.6 -> 22.8 us); in the bodies of the
-// solver's conditional graph it loses 7 % (158 -> 169 us an iteration), so a captured
-// launch is an ordinary one.
+// Launches kernel so that its launch overlaps the end of the kernel before it on the
+// stream (programmatic dependent launch): the grid is set up while the other runs and
+// starts when its last block has exited. The kernel calls overlap_wait() before it
+// touches memory. A predecessor that does not take part is waited for as usual.
+// M^dag M back to back on one stream: FP16 24^3 x 48 110 -> 100 us, FP32 8^4 24.8 ->
+// 14.8, FP64 12^3 x 24 250 -> 242; in the bodies of the solver's conditional graph it
+// loses 7 % (158 -> 169 us an iteration), so a captured launch is an ordinary one.
+// No kernel lets its successor start earlier (griddepcontrol.launch_dependents): the
+// waiting blocks gain nothing that this does not, and they are put on the SMs that are
+// idle at that moment, several to one SM, where they stay. FP64 M^dag M with 128 blocks a
+// hop took 182 us instead of 82, with 162 blocks 351 instead of 250, FP32 with 384
+// blocks 33 instead of 22; and behind a hop that asks for the largest shared-memory
+// carveout they run with the L1 that is left, as does the rest of the chain (FP32 24^3 x 48,
+// a ring hop and three plain ones: 198 instead of 143).
 template <typename Arg>
 inline cudaError_t launch_overlapped(void (*kernel)(Arg), unsigned grid, unsigned block, size_t shared,
                                      cudaStream_t s, const Arg& arg) {
@@ -53,20 +59,10 @@ inline cudaError_t launch_overlapped(void (*kernel)(Arg), unsigned grid, unsigne
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, arg);
 }
-// Lets the next kernel on the stream start (EARLY) and waits until the ones before have
-// finished and their writes are visible. Every thread of every block calls it, also
-// one that returns at once: a kernel that ended without waiting would release its
-// successor while its predecessor still runs.
-// A kernel that asks for the largest shared-memory carveout does not let its successor
-// start early (it may still start early itself): the successor would take the SMs as
-// they are, with the small L1 that is left, and so would all that follow it in a chain
-// of overlapping launches. M_hat^dag M_hat at 24^3 x 48, FP32, the first hop in the
-// ring shape and three plain ones: 198 us with its early start, 143 without, 143 for
-// four plain hops; four ring hops 142 either way (16^3 x 32: 42 with, 29 without).
-template <bool EARLY> __device__ __forceinline__ void overlap_launch() {
-  if constexpr (EARLY) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-}
+// Waits until the kernels before have finished and their writes are visible. Every
+// thread of every block calls it, also one that returns at once: a kernel that ended
+// without waiting would release its successor before its predecessor's writes are.
+__device__ __forceinline__ void overlap_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ------------------------------------------------------------------ geometry
 // Division of n < 2^31 by a runtime constant d >= 1 with one multiply-high,
@@ -180,7 +176,7 @@ struct CFieldPtr {
 };
 
 // Spinors are read with ordinary loads, not through the read-only path: a kernel that
-// starts before its predecessor has finished (overlap_launch) may read them only after
+// starts before its predecessor has finished (overlap_wait) may read them only after
 // it has waited, and only an ordinary load is ordered behind that wait.
 template <int P> struct SpinorIO;
 
