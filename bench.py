@@ -662,16 +662,17 @@ def hop_roofline(L, F, lat, gsl, prec, flush, stream, vh, launches=40):
 HOP_SHAPE_MEANING = {0: "128 threads, one site per thread", 1: "128 threads, one site per thread, <= 72 registers",
                      2: "128 threads, one site per thread, spin components paired in packed FP32x2 arithmetic, "
                         "<= 72 registers",
-                     3: "128 threads, one site per thread, links and neighbours staged in shared memory when n5 >= 4, "
-                        "spin-paired packed FP32x2 arithmetic, <= 64 registers",
-                     4: "as 3, <= 72 registers",
+                     3: "128 threads, one site per thread, <= 96 registers",
+                     4: "128 threads, one site per thread, links and neighbours staged in shared memory when n5 >= 4, "
+                        "spin-paired packed FP32x2 arithmetic, <= 72 registers",
                      5: "128 threads, one site per thread, links and neighbours staged in shared memory when n5 >= 4, "
                         "<= 72 registers",
                      6: "128 threads, one site per thread, spin components paired in packed FP32x2 arithmetic",
                      7: "128 threads, one site per thread, <= 72 registers, neighbour spinors and links copied "
                         "asynchronously (cp.async) through a shared-memory ring",
                      8: "128 threads, one site per thread, spin-paired packed FP32x2 arithmetic, <= 72 registers, "
-                        "neighbour data copied asynchronously through a shared-memory ring"}
+                        "neighbour data copied asynchronously through a shared-memory ring",
+                     9: "as 4, <= 64 registers"}
 
 
 def hop_key(prec, recon, dagger, epi, red, dims, n5, full=0):

@@ -385,8 +385,9 @@ int lqcd_batch_cg_solve(int n, const lqcd_batch_item* items, int recon, const lq
  *    threads and at least 7 resident blocks per SM; 2: as 6 with at least 7
  *    blocks per SM; 5: 128 threads, one site per thread, at least 7 blocks per
  *    SM, the eight links and neighbours of each 4D site staged once in shared
- *    memory for its n5 threads when n5 >= 4 (shape 0 otherwise); 4 / 3: as 5
- *    with the arithmetic of 6, at least 7 / 8 blocks per SM;
+ *    memory for its n5 threads when n5 >= 4 (shape 0 otherwise); 4 / 9: as 5
+ *    with the arithmetic of 6, at least 7 / 8 blocks per SM; 3: as 1 with
+ *    at least 5 blocks per SM;
  *    6: 128 threads, one site per thread, the two spin components of each
  *    half spinor paired in packed FP32x2 arithmetic; 7 / 8: as 1 / 2 with
  *    each direction's neighbour spinor and link copied asynchronously into a

@@ -32,21 +32,23 @@ constexpr int HOP_BLOCK = 128;
 // shared memory once per 4D site for its n5 threads (L_s-replicated and multi-RHS
 // hops, n5 >= 4; otherwise shape 0).
 // Measured on GB300, M_hat^dag M_hat: 24^3 x 48 FP16 / 12-real, shapes 0, 1, 2, 6, 7, 8:
-// 101, 100, 100, 104, 99, 99 us (latency and the tail of 2.4 waves bound every form
-// there; 110 without overlapped launches). 32^4 with 12 RHS, FP16: 1,434 (shape 0),
-// 1,411 (2), 1,239 (5), 1,217 (4), 1,186 (3); FP32: 1,729 (1), 1,606 (5), 1,681 (4),
-// 1,658 (3). Domain wall 16^4 x 16, FP32: 173 (2), 160 (5), 161 (4), 167 (3). Staging
+// 101, 101, 99, 106, 100, 100 us (latency and the tail of 2.4 waves bound every form
+// there; 110 without overlapped launches); FP32 / 18-real, whose nine loads per link want
+// registers, without overlap: 242, 232, 201, 230, 223, 218, and 191 in shape 3 (20^3 x 40:
+// 101 against 119 in the next best). 32^4 with 12 RHS, FP16: 1,434 (shape 0),
+// 1,411 (2), 1,239 (5), 1,217 (4), 1,186 (9); FP32: 1,729 (1), 1,606 (5), 1,681 (4),
+// 1,658 (9). Domain wall 16^4 x 16, FP32: 173 (2), 160 (5), 161 (4), 167 (9). Staging
 // takes 35 % of the instructions out (445 -> 278 million warp instructions a hop for
 // 12 RHS); what is left waits for loads, so that resident warps pay even at the price
 // of some spilled registers (5, 6, 7, 8 blocks per SM, FP16: 1,321, 1,255, 1,219, 1,186).
 // Shape 0 is the default; the tuner times all of them per key.
-#define LQCD_HOP_SHAPES(X) X(0, 128, 1, 0) X(1, 128, 1, 7) X(2, 128, -2, 7) X(3, 128, -5, 8) X(4, 128, -5, 7) \
-  X(5, 128, -1, 7) X(6, 128, -2, 0) X(7, 128, -3, 7) X(8, 128, -4, 7)
-constexpr int HOP_SHAPES = 9;
+#define LQCD_HOP_SHAPES(X) X(0, 128, 1, 0) X(1, 128, 1, 7) X(2, 128, -2, 7) X(3, 128, 1, 5) X(4, 128, -5, 7) \
+  X(5, 128, -1, 7) X(6, 128, -2, 0) X(7, 128, -3, 7) X(8, 128, -4, 7) X(9, 128, -5, 8)
+constexpr int HOP_SHAPES = 10;
 // Raised whenever an index comes to mean another kernel: saved tables carry it.
-constexpr int HOP_SHAPES_VERSION = 2;
+constexpr int HOP_SHAPES_VERSION = 3;
 // Whether shape i differs from shape 0 for n5 slices (the tuner skips it otherwise).
-inline bool hop_shape_applies(int i, int n5) { return (i != 3 && i != 4 && i != 5) || n5 >= STAGE_MIN_N5; }
+inline bool hop_shape_applies(int i, int n5) { return (i != 4 && i != 5 && i != 9) || n5 >= STAGE_MIN_N5; }
 // The shape used when the table holds no choice for a hop.
 constexpr int HOP_SHAPE_DEFAULT = 0;
 
