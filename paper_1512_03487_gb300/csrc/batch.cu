@@ -398,7 +398,7 @@ struct BatchSolver : CgEngine {
   }
 };
 
-static int sm_count(int* sms) {
+int sm_count(int* sms) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);

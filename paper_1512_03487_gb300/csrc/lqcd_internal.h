@@ -17,6 +17,9 @@ int launch_hop_f16(int recon, bool dagger, int epi, int reduce, HopArgs a, cudaS
 int launch_hop_gparity(int prec, int recon, bool dagger, int epi, int reduce, HopArgs a, cudaStream_t s);
 int launch_hop_df(int recon, bool dagger, int epi, int reduce, HopArgs a, cudaStream_t s);
 
+// Multiprocessors of the current device.
+int sm_count(int* sms);
+
 // Threads per block of the one-site hop (FP64, G-parity, the batch solver's tiles).
 // Every hop launch shape covers at least 64 sites per block: the solvers size
 // their reduction partials for that.

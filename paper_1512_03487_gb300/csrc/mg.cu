@@ -273,11 +273,13 @@ __device__ __forceinline__ bool sum_finite(double) { return true; }  // FP64 sum
 // vectors at a time give 16 terms per thread (two chiralities, real and imaginary)
 // that go to shared memory; then each thread adds up 16 of them.
 // 24^3 x 48, 12 FP32 vectors, 4^4 aggregates on GB300: 516 -> 171 us, 0.72 of the
-// measured copy bandwidth.
+// measured copy bandwidth. With fewer aggregates than fill the SMs a block takes only
+// `per` vectors (blockIdx.y the next ones): 24 FP64 vectors on 16 aggregates of 4^4 took 89 us
+// in 16 blocks, 23 with a block per vector and aggregate.
 constexpr int RS_BLOCK = 256;
 template <int P, int B>
 __global__ void __launch_bounds__(RS_BLOCK, P == LQCD_F32 ? 4 : 1) k_restrict(void* coarse, const void* fine,
-                                                                              const void* vecs, MGGeom m) {
+                                                                              const void* vecs, MGGeom m, int per) {
   using T = typename PrecTraits<P>::real;
   using S = typename SumOf<T>::type;
   constexpr int SITES = B * B * B * B;
@@ -297,12 +299,13 @@ __global__ void __launch_bounds__(RS_BLOCK, P == LQCD_F32 ? 4 : 1) k_restrict(vo
   // 4^4: thread t sums value t / 16 over the sites t % 16 + 16 i and meets 15 others;
   // 2^4: thread t sums value t % 16 of its aggregate t / 16
   const int val = B == 4 ? tid >> 4 : tid & 15, start = B == 4 ? tid & 15 : tid & ~15, stride = B == 4 ? 16 : 1;
-  for (int k0 = 0; k0 < m.nv; k0 += 4) {
-    T* buf = sh[BUFS == 2 ? (k0 >> 2) & 1 : 0];
+  const int first = blockIdx.y * per, end = first + per < m.nv ? first + per : m.nv;
+  for (int k0 = first; k0 < end; k0 += 4) {
+    T* buf = sh[BUFS == 2 ? ((k0 - first) >> 2) & 1 : 0];
 #pragma unroll 1  // one vector's registers: 32 warps per SM keep more loads in flight than unrolling does
     for (int q = 0; q < 4; q++) {
       T re[2] = {T(0), T(0)}, im[2] = {T(0), T(0)};
-      if (k0 + q < m.nv) {
+      if (k0 + q < end) {
         Spinor<T> v;
         SpinorIO<P>::load(fine_ptr<P>(vecs, m, k0 + q, parity), m.g.sstride, cb, v);
 #pragma unroll
@@ -334,7 +337,7 @@ __global__ void __launch_bounds__(RS_BLOCK, P == LQCD_F32 ? 4 : 1) k_restrict(vo
     if (P == LQCD_F32 && __any_sync(0xffffffffu, !sum_finite(s))) sum = total(0.0);
     // value: vector k0 + val / 4, chirality (val / 2) % 2, real or imaginary part
     const int k = k0 + (val >> 2);
-    if (act && k < m.nv && (B == 2 || (tid & 15) == 0))
+    if (act && k < end && (B == 2 || (tid & 15) == 0))
       out[(agg * m.nc + ((val >> 1) & 1) * m.nv + k) * 2 + (val & 1)] = (T)sum;
   }
 }
@@ -420,6 +423,7 @@ __device__ __forceinline__ void coarse_row(const Piece<T>* y, int64_t ystep, con
 #pragma unroll
       for (int p = 0; p < NP; p++) add(y[p * CA_LANES], v[p * CA_LANES]);
     } else {
+#pragma unroll 4
       for (int p = 0; p + l < pieces; p += CA_LANES) add(y[p], v[p]);
     }
     sr = add_term(sr, r);
@@ -462,13 +466,14 @@ __global__ void __launch_bounds__(MG_BLOCK) k_coarse_apply(cpx<T>* out, const cp
   if (l == 0 && i < nc) out[(int64_t)X * nc + i] = mk((T)re, (T)im);
 }
 
-// The adjoint, out(X)_i = sum_d sum_j conj(Y_{-d}(X + d)_ji) in(X + d)_j, from the
-// blocks as they are stored (the solver keeps the adjoint stencil's own blocks
-// and uses k_coarse_apply). One warp per (coarse site, row): the lanes take the
-// 9 Nc products in turn and the warp sums them.
-template <typename T>
-__global__ void __launch_bounds__(MG_BLOCK) k_coarse_apply_dag(cpx<T>* out, const cpx<T>* in, const cpx<T>* Y,
-                                                               MGGeom m) {
+// One warp per (coarse site, row): the lanes take the 9 Nc products in turn and the warp
+// sums them. For the adjoint, out(X)_i = sum_d sum_j conj(Y_{-d}(X + d)_ji) in(X + d)_j
+// from the blocks as they are stored (the solver keeps the adjoint stencil's own blocks
+// and uses k_coarse_apply), and where that kernel's four lanes per row leave too much to
+// each lane (row_per_warp).
+template <typename T, bool DAG>
+__global__ void __launch_bounds__(MG_BLOCK) k_coarse_apply_warp(cpx<T>* out, const cpx<T>* in, const cpx<T>* Y,
+                                                                MGGeom m) {
   const int64_t wid = ((int64_t)blockIdx.x * MG_BLOCK + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (wid >= m.Vc * m.nc) return;  // whole warps exit together
@@ -502,7 +507,8 @@ __global__ void __launch_bounds__(MG_BLOCK) k_coarse_apply_dag(cpx<T>* out, cons
     const int j = q - d * nc;
     const cpx<T> v = in[(int64_t)Xn * nc + j];
     const int dr = d == 0 ? 0 : (((d - 1) ^ 1) + 1);  // opposite direction
-    const cpx<T> y = conj(Y[(((int64_t)dr * m.Vc + Xn) * nc + j) * nc + i]);
+    const cpx<T> y = DAG ? conj(Y[(((int64_t)dr * m.Vc + Xn) * nc + j) * nc + i])
+                         : Y[(((int64_t)d * m.Vc + X) * nc + i) * nc + j];
     const cpx<T> p = cmul(y, v);
     if (sizeof(T) == 8) {
       dr_ += (double)p.r;
@@ -793,8 +799,16 @@ template <typename F> static int dispatch_prec(int prec, F&& f) {
 static int restrict_(const MGGeom& m, int prec, void* coarse, const void* fine, const void* vecs, cudaStream_t s) {
   return dispatch_prec(prec, [&](auto P) {
     constexpr int PR = decltype(P)::value;
-    if (m.b == 4) k_restrict<PR, 4><<<(unsigned)m.Vc, RS_BLOCK, 0, s>>>(coarse, fine, vecs, m);
-    else k_restrict<PR, 2><<<(unsigned)((m.Vc + 15) / 16), RS_BLOCK, 0, s>>>(coarse, fine, vecs, m);
+    int sms = 0, st = sm_count(&sms);
+    if (st) return st;
+    // fewer blocks than SMs: fewer vectors to a block, until two blocks per SM have work
+    const int64_t groups = m.b == 4 ? m.Vc : (m.Vc + 15) / 16;
+    int per = (m.nv + 3) / 4 * 4;
+    while (groups < sms && per > 1 && groups * ((m.nv + per - 1) / per) < 2 * sms)
+      per = per > 4 ? (per / 2 + 3) / 4 * 4 : per / 2;
+    const dim3 grid((unsigned)groups, (unsigned)((m.nv + per - 1) / per));
+    if (m.b == 4) k_restrict<PR, 4><<<grid, RS_BLOCK, 0, s>>>(coarse, fine, vecs, m, per);
+    else k_restrict<PR, 2><<<grid, RS_BLOCK, 0, s>>>(coarse, fine, vecs, m, per);
     return after_launch("k_restrict");
   });
 }
@@ -805,13 +819,26 @@ static int prolong_(const MGGeom& m, int prec, void* fine, const void* coarse, c
     return after_launch("k_prolong");
   });
 }
+// Where a warp per row beats k_coarse_apply's four lanes per row: too few rows to fill the
+// SMs with four lanes each, and rows of one vector or, in FP64, of an odd number below
+// eight (2, 6, 10, 14 pieces, few and unequal per lane). GB300, us, four lanes / warp:
+// FP64, 16 sites, 24 vectors 31.3 / 10.7; 256 sites, 8 vectors 13.1 / 13.9, 12 vectors 17.7 /
+// 24.8; 1,296 sites, 3 vectors 20.1 / 13.8, 7 vectors 55 / 39; 10,000 sites, 3 vectors 83 / 83,
+// 6 vectors 150 / 246. FP32, 16 sites, 24 vectors 10.9 / 6.4; 256 sites, 7 vectors 6.5 / 4.1,
+// 12 vectors 6.4 / 8.0; 1,296 sites, 2 vectors 5.3 / 4.2; 10,000 sites, one vector 12.7 / 7.8,
+// two 12.8 / 16.8.
+static bool row_per_warp(const MGGeom& m, bool f64) {
+  return m.nv == 1 || (f64 && m.nv % 2 == 1 && m.nv < 8) || m.Vc * m.nc < (m.nv == 2 ? 8192 : 4096);
+}
 template <typename T>
 static void launch_coarse_apply(const MGGeom& m, void* out, const void* in, const void* Y, int dagger, cudaStream_t s) {
-  const int64_t warps = dagger ? m.Vc * m.nc : m.Vc * ((m.nc * CA_LANES + 31) / 32);
+  const bool wide = dagger || row_per_warp(m, sizeof(T) == 8);
+  const int64_t warps = wide ? m.Vc * m.nc : m.Vc * ((m.nc * CA_LANES + 31) / 32);
   auto* o = static_cast<cpx<T>*>(out);
   auto* i = static_cast<const cpx<T>*>(in);
   auto* y = static_cast<const cpx<T>*>(Y);
-  if (dagger) k_coarse_apply_dag<T><<<n_grid(warps * 32), MG_BLOCK, 0, s>>>(o, i, y, m);
+  if (dagger) k_coarse_apply_warp<T, true><<<n_grid(warps * 32), MG_BLOCK, 0, s>>>(o, i, y, m);
+  else if (wide) k_coarse_apply_warp<T, false><<<n_grid(warps * 32), MG_BLOCK, 0, s>>>(o, i, y, m);
   else {
     const int pieces = m.nc * (int)sizeof(cpx<T>) / 16;
     const unsigned grid = n_grid(warps * 32);

@@ -73,10 +73,10 @@ def test_restrict_partial_sums_beyond_the_range(L, b, axis, sign):
     assert got[0].imag == 0 and got[1] == 0
 
 
-@pytest.mark.parametrize("nv", [1, 2, 3, 12, 28])
+@pytest.mark.parametrize("nv,dims", [(1, (8, 4, 2, 4)), (2, (8, 4, 2, 4)), (12, (8, 4, 2, 4)),  # a warp per row
+                                     (3, (16, 16, 8, 8)), (4, (16, 16, 8, 8)), (12, (8, 8, 8, 6)), (28, (8, 8, 8, 4))])
 @pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
-def test_coarse_apply_carries_values_that_are_not_finite(L, nv, value):
-    dims = (8, 4, 2, 4)
+def test_coarse_apply_carries_values_that_are_not_finite(L, nv, dims, value):
     lat, cd, rng = L.lattice(dims), tuple(d // 2 for d in dims), make_rng(2511 + nv)
     Y = _f32(rng.standard_normal((9,) + cd[::-1] + (2 * nv, 2 * nv, 2)) @ np.array([1.0, 1j]))
     c = _f32(rng.standard_normal(cd[::-1] + (2 * nv, 2)) @ np.array([1.0, 1j]))
@@ -93,12 +93,13 @@ def test_coarse_apply_carries_values_that_are_not_finite(L, nv, value):
               part(Y.real, c.imag) + part(Y.imag, c.real))
 
 
+@pytest.mark.parametrize("nv,dims", [(1, (2, 2, 2, 2)), (3, (16, 16, 8, 8))])
 @pytest.mark.parametrize("sign", [1.0, -1.0])
-def test_coarse_apply_sums_beyond_the_range(L, sign):
-    """Nine blocks of products 1e38 each: the sum leaves FP32's range, with its sign."""
-    lat = L.lattice((2, 2, 2, 2))
-    c = torch.full((2,), sign * 5e37, dtype=torch.complex64, device="cuda")
-    Y = torch.ones((9, 2, 2), dtype=torch.complex64, device="cuda")
-    out = torch.zeros(2, dtype=torch.complex64, device="cuda")
-    L.lqcd_mg_coarse_apply(out, c, Y, 1, 2, 1, 0, lat)
+def test_coarse_apply_sums_beyond_the_range(L, nv, dims, sign):
+    """Nine blocks of products 5e37 each: the sum leaves FP32's range, with its sign."""
+    lat, sites, nc = L.lattice(dims), int(np.prod(dims)) // 16, 2 * nv
+    c = torch.full((sites * nc,), sign * 5e37, dtype=torch.complex64, device="cuda")
+    Y = torch.ones(9 * sites * nc * nc, dtype=torch.complex64, device="cuda")
+    out = torch.zeros(sites * nc, dtype=torch.complex64, device="cuda")
+    L.lqcd_mg_coarse_apply(out, c, Y, nv, 2, 1, 0, lat)
     assert (out.cpu().numpy().real == sign * np.inf).all()
