@@ -85,7 +85,7 @@ __device__ __forceinline__ bool site_of_thread(const Geom& g, int64_t t, int& pa
 // instruction occupies its SM quarter for 64 cycles), so the work is cut down to
 // the fewest FP64 instructions and split finely enough that every SM gets the
 // same share; the links come from L1 / L2 and memory is nearly idle. 16^4 on
-// GB300, before and after: gauge force 817 -> 570 us, link update 1,058 -> 253 us,
+// GB300, before and after: gauge force 817 -> 570 us, link update 1,058 -> 149 us,
 // plaquette 209 -> 170 us.
 
 constexpr int PLAQ_SITES = 64;  // sites per block; two warps each take three of the six planes of 32 sites
