@@ -33,7 +33,8 @@ inline int64_t round_up(int64_t a, int64_t b) { return (a + b - 1) / b * b; }
 // touches memory. A predecessor that does not take part is waited for as usual.
 // M^dag M back to back on one stream: FP16 24^3 x 48 110 -> 100 us, FP32 8^4 24.8 ->
 // 14.8, FP64 12^3 x 24 250 -> 242; in the bodies of the solver's conditional graph it
-// loses 7 % (158 -> 169 us an iteration), so a captured launch is an ordinary one.
+// gains nothing (24^3 x 48 FP16 140-142 us an iteration, 12^3 x 24 FP32 32 either way),
+// so a captured launch is an ordinary one.
 // No kernel lets its successor start earlier (griddepcontrol.launch_dependents): the
 // waiting blocks gain nothing that this does not, and they are put on the SMs that are
 // idle at that moment, several to one SM, where they stay. FP64 M^dag M with 128 blocks a
